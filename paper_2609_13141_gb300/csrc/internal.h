@@ -37,7 +37,7 @@ struct KernelEnv {
 
 // ---- tcgen05 GEMM:  C[b] = epi(A[b] @ B[b % b_mod]^T (+ bias)), bf16 out (the MLP).
 // A: [batches][M][K], B: [nb][N][K], C: [batches][M][ldc] (row stride ldc).
-// N must be a multiple of bn (64, 128 or 256), K a multiple of 64.
+// N and K must be multiples of 64.
 struct GemmProblem {
     const void* A;
     const void* B;
@@ -48,7 +48,7 @@ struct GemmProblem {
     long long c_batch_stride;
     int ldc;
     int gelu;            // 1: exact-erf GELU epilogue
-    int bn;              // 64, 128 or 256
+    int after_gemm;      // 1: A is written by the launch_gemm just before on the stream (launched ahead of its end)
     int max_ctas;        // persistent grid size cap (0: one per SM)
 };
 cudaError_t launch_gemm(const GemmProblem& p, const KernelEnv& env, const char** err);
