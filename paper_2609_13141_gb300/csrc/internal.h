@@ -24,8 +24,9 @@ int make_tmap_bf16_3d(CUtensorMap* map, const void* base, uint64_t inner, uint64
 // the record and call nothing (so a launch inside a stream capture that was
 // preceded by one outside it sets nothing).  Thread-safe.
 // max_carveout also asks for the largest shared-memory carveout (L1 shrinks to
-// what is left), for kernels that need it to fit several CTAs on an SM.
-cudaError_t ensure_smem_attr(const void* func, size_t bytes, bool max_carveout = false);
+// what is left), for kernels that need it to fit several CTAs on an SM;
+// big_clusters allows clusters of more than eight CTAs.
+cudaError_t ensure_smem_attr(const void* func, size_t bytes, bool max_carveout = false, bool big_clusters = false);
 // Multiprocessor count of the current device (cached per device, thread-safe).
 int device_sm_count();
 
@@ -171,10 +172,12 @@ struct DecodeArgs {
     int* cnt_attn;              // [B*Hkv]
     int nsplit_s;               // score CTAs per group (kDecScoreChunk blocks each)
     int nsplit_a, bpc, nst;     // attention CTAs per group, list entries per CTA, ring stages
+    int cluster;                // 1: a group's attention CTAs form one cluster and merge among themselves
 };
 constexpr int kDecScoreChunk = 256;
-// Attention split for a group list of at most max_len entries.
-void decode_attn_split(int max_len, int d, int* nsplit, int* bpc, int* nst);
+// Attention split for `groups` lists of at most max_len entries on sms SMs.
+void decode_attn_split(int max_len, int d, bool dense, int groups, int sms, int* nsplit, int* bpc, int* nst,
+                       int* cluster);
 // Dynamic shared memory the score and attention kernels need.
 size_t decode_score_smem(int nsplit, int topk, int d_sel);
 size_t decode_attn_smem(int d, int G, int nst, int bpc);

@@ -10,21 +10,23 @@
 //                      staged in shared memory by bulk async copies.  Each CTA keeps
 //                      the exact Top-K of its own blocks (rank by counting); the
 //                      last CTA of a group selects the Top-K of those candidates
-//                      (step 2) by a radix select on the scores' order-preserving
-//                      bit patterns, ties to the lower block, and writes the kept
-//                      list in ascending order.
-//   dec_attn_kernel    split-KV attention over B_0 and the kept blocks (steps 3-4):
-//                      each CTA streams one or a few pages (K and V slices of 16 KB
-//                      at d = 128, bulk async copies into a ring), keeps an online
-//                      softmax per head, and the last CTA of a group merges the
-//                      partial (max, sum, output) triples.
+//                      (step 2) on the scores' order-preserving bit patterns, by
+//                      counting ranks or, past 512 candidates, a radix select, ties to
+//                      the lower block, and writes the kept list in ascending order.
+//   dec_attn_tc_kernel split-KV attention over B_0 and the kept blocks (steps 3-4),
+//                      d = 128: each CTA takes a few pages (K and V slices of 16 KB,
+//                      TMA into a ring), two pages a step on the tensor cores, and
+//                      keeps an online softmax per head.  A SAS list's CTAs form a
+//                      cluster and merge their partial (max, sum, output) triples
+//                      over distributed shared memory; a dense list's last CTA merges
+//                      them from global memory.
+//   dec_attn_kernel    the same for d = 64 on the CUDA cores.
 // The three kernels are chained with programmatic dependent launch: each one
 // starts while its predecessor runs, does the work that needs none of the
-// predecessor's results (barrier set-up, reading lengths and queries, the page
-// of the current block) and then waits on the grid dependency.
-// A decode step moves bytes, not flops (a few FMAs per cached element), so the
-// arithmetic runs on CUDA cores with packed fp32x2 FMAs; there is no tensor-core
-// contraction on this path.
+// predecessor's results (barrier set-up, reading lengths and queries, the block
+// summaries, the page of the current block) and then waits on the grid dependency.
+// A decode step moves bytes, not flops, and is bound by latencies: at 8 sequences
+// of 64K tokens (8 KV heads, K = 32) 39.8 us a step, against 12.6 us for its bytes.
 #include <math_constants.h>
 
 #include "internal.h"
@@ -39,6 +41,7 @@ constexpr int kPrepThreads = 256;
 constexpr int kScoreThreads = 256;
 constexpr int kAttnThreads = 256;
 constexpr int kStages = 3;
+constexpr int kRankMax = 512;         // candidates ranked by counting (M^2 comparisons); more take the radix select
 constexpr float kLog2e = 1.4426950408889634f;
 
 __device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
@@ -91,42 +94,60 @@ __device__ int block_excl_scan(int v, int* scan) {
 
 // One full block's summary (App. B): the mean of its 64 keys in fp32, projected
 // by the KV head's Wk [d_sel][d] and rounded to bf16.  256 threads.
-// red: 512 floats, kbar: 128 floats of shared memory.
-__device__ void summarize_block(const bf16* Kt, const bf16* Wk, bf16* out, int d, int d_sel, float* red,
-                                float* kbar) {
-    const int t = threadIdx.x;
-    const int nw = d >> 1;                    // bf16 pairs per key row
-    const int groups = kPrepThreads / nw;     // 4 (d = 128) or 8 (d = 64) row groups
-    const int rows = kBlk / groups;
-    const int wi = t % nw, rg = t / nw;
+// red: 512 floats, kbar: 128 floats of shared memory.  Latency: a thread's key
+// words and its warp's rows of Wk are all requested before the first is used
+// (loaded one by one they made a step that closes a block wait 11 us on this).
+template <int D>
+__device__ void summarize_block_d(const bf16* Kt, const bf16* Wk, bf16* out, int d_sel, float* red, float* kbar) {
+    constexpr int NW = D / 2;                    // bf16 pairs per key row
+    constexpr int GROUPS = kPrepThreads / NW;    // 4 (d = 128) or 8 (d = 64) row groups
+    constexpr int ROWS = kBlk / GROUPS;
+    constexpr int OUTS = 128 / (kPrepThreads / 32);   // projection rows per warp, at most
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int wi = t % NW, rg = t / NW;
     const uint32_t* K32 = reinterpret_cast<const uint32_t*>(Kt);
-    float a0 = 0.f, a1 = 0.f;
-    for (int r = rg * rows; r < (rg + 1) * rows; ++r) {
-        const uint32_t w = __ldg(K32 + r * nw + wi);
-        a0 += bf_lo(w);
-        a1 += bf_hi(w);
+    uint32_t kw[ROWS], ww[OUTS][NW / 32];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) kw[r] = __ldg(K32 + (rg * ROWS + r) * NW + wi);
+#pragma unroll
+    for (int k = 0; k < OUTS; ++k) {
+        const int o = warp + k * (kPrepThreads / 32);
+        const uint32_t* row = reinterpret_cast<const uint32_t*>(Wk + static_cast<size_t>(o) * D);
+#pragma unroll
+        for (int e = 0; e < NW / 32; ++e) ww[k][e] = o < d_sel ? __ldg(row + e * 32 + lane) : 0u;
     }
-    red[rg * d + 2 * wi] = a0;
-    red[rg * d + 2 * wi + 1] = a1;
+    float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        a0 += bf_lo(kw[r]);
+        a1 += bf_hi(kw[r]);
+    }
+    red[rg * D + 2 * wi] = a0;
+    red[rg * D + 2 * wi + 1] = a1;
     __syncthreads();
-    if (t < d) {
+    if (t < D) {
         float s = 0.f;
-        for (int g = 0; g < groups; ++g) s += red[g * d + t];
+        for (int g = 0; g < GROUPS; ++g) s += red[g * D + t];
         kbar[t] = s * (1.f / kBlk);
     }
     __syncthreads();
-    const int warp = t >> 5, lane = t & 31;
-    for (int o = warp; o < d_sel; o += kPrepThreads / 32) {
-        const uint32_t* row = reinterpret_cast<const uint32_t*>(Wk + static_cast<size_t>(o) * d);
+#pragma unroll
+    for (int k = 0; k < OUTS; ++k) {
+        const int o = warp + k * (kPrepThreads / 32);
         float acc = 0.f;
-        for (int e = lane; e < nw; e += 32) {
-            const uint32_t w = __ldg(row + e);
-            acc = fmaf(bf_lo(w), kbar[2 * e], acc);
-            acc = fmaf(bf_hi(w), kbar[2 * e + 1], acc);
+#pragma unroll
+        for (int e = 0; e < NW / 32; ++e) {
+            acc = fmaf(bf_lo(ww[k][e]), kbar[2 * (e * 32 + lane)], acc);
+            acc = fmaf(bf_hi(ww[k][e]), kbar[2 * (e * 32 + lane) + 1], acc);
         }
         acc = warp_sum(acc);
-        if (lane == 0) out[o] = __float2bfloat16_rn(acc);
+        if (lane == 0 && o < d_sel) out[o] = __float2bfloat16_rn(acc);
     }
+}
+__device__ void summarize_block(const bf16* Kt, const bf16* Wk, bf16* out, int d, int d_sel, float* red,
+                                float* kbar) {
+    if (d == 128) summarize_block_d<128>(Kt, Wk, out, d_sel, red, kbar);
+    else summarize_block_d<64>(Kt, Wk, out, d_sel, red, kbar);
 }
 
 // grid (B*Hkv, 1 + d_sel/8): y = 0 appends the token and updates the summary
@@ -242,20 +263,21 @@ __global__ void __launch_bounds__(kPrepThreads) dec_summarize_kernel(DecodeArgs 
 
 struct ScoreSmem {
     size_t r0;   // staged summary rows; in the last CTA the candidates (keys, blocks)
-    size_t qs, bars, misc, xchg, hist, scan, total;
+    size_t qs, bars, misc, xchg, scan, hist, total;
 };
 __host__ __device__ inline ScoreSmem score_smem_layout(int nsplit, int topk, int d_sel) {
     ScoreSmem L;
     const size_t slab = static_cast<size_t>(8) * 32 * d_sel * 2;
-    const size_t cand = static_cast<size_t>(nsplit) * (topk > 0 ? topk : 1) * 8;
+    const size_t cand = (static_cast<size_t>(nsplit) * (topk > 0 ? topk : 1) + 4) * 8;
     L.r0 = ((slab > cand ? slab : cand) + 127) / 128 * 128;
     L.qs = L.r0;                  // d_sel bf16 (<= 256 bytes)
     L.bars = L.qs + 256;          // 8 mbarriers
     L.misc = L.bars + 64;         // flag, radix broadcast, per-warp counts (16 ints)
-    L.xchg = L.misc + 64;         // 256 64-bit sort keys
-    L.hist = L.xchg + 256 * 8;    // 4096 ints
-    L.scan = L.hist + 4096 * 4;   // 16 ints
-    L.total = L.scan + 128;
+    L.xchg = L.misc + 64;         // 256 order keys
+    L.scan = L.xchg + 256 * 4;    // 16 ints
+    L.hist = L.scan + 128;        // 4096 ints of the radix select; kept for every size: two CTAs an
+                                  // SM run a step of 8 x 64K in 39.8 us, three (without them) in 44.3
+    L.total = L.hist + 4096 * 4;
     return L;
 }
 
@@ -267,29 +289,54 @@ __device__ __forceinline__ uint32_t order_key(float f) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// Descending bitonic sort of 256 distinct 64-bit keys, one per thread of the
-// CTA; returns the key that ends at position threadIdx.x.  Exchanges within a
-// warp use shuffles, wider ones the 256-entry shared buffer xchg.
-__device__ uint64_t bitonic256_desc(uint64_t c, uint64_t* xchg) {
-    const int t = threadIdx.x;
-#pragma unroll
-    for (int k = 2; k <= 256; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            uint64_t o;
-            if (j >= 32) {
-                xchg[t] = c;
-                __syncthreads();
-                o = xchg[t ^ j];
-                __syncthreads();
-            } else {
-                o = __shfl_xor_sync(0xffffffffu, c, j);
-            }
-            const bool keep_max = ((t & j) == 0) == ((t & k) == 0);
-            c = keep_max ? (c > o ? c : o) : (c < o ? c : o);
-        }
+// How many of the M keys (16-byte aligned, the rest of the last four slots 0) rank
+// ahead of key (>= 1) at position t: the larger ones, and the equal ones listed
+// before it.  All lanes of a warp read the same four keys at a time; the
+// position decides only for keys in the warp's own range, w0 .. w0 + 31.
+__device__ __forceinline__ int rank_of(const uint32_t* keys, int M, uint32_t key, int t, int w0) {
+    int r = 0;
+    for (int j = 0; j < M; j += 4) {
+        const uint4 k4 = *reinterpret_cast<const uint4*>(keys + j);
+        // an equal key ranks ahead when listed before: compare with key - 1 there
+        const bool own = j >= w0 && j < w0 + 32;
+        const uint32_t all = key - (j < w0 ? 1u : 0u);
+        r += k4.x > (own ? key - (j < t) : all);
+        r += k4.y > (own ? key - (j + 1 < t) : all);
+        r += k4.z > (own ? key - (j + 2 < t) : all);
+        r += k4.w > (own ? key - (j + 3 < t) : all);
     }
-    return c;
+    return r;
+}
+
+// Exact Top-K of at most 512 candidates in ascending block order by counting each
+// one's rank (M^2 comparisons, about 1 us at 160 candidates, against 4 us of the
+// radix select's three histogram passes); same arguments as select_candidates.
+__device__ void select_by_rank(const DecodeArgs& a, int bh, int M, const uint32_t* keys, const int32_t* idx,
+                               int* scan) {
+    const int K = a.topk, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    int32_t* lst = a.list + static_cast<size_t>(bh) * 64;
+    int32_t* so = a.sel_idx ? a.sel_idx + static_cast<size_t>(bh) * K : nullptr;
+    bool take[2];
+    unsigned bal[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int i = h * kScoreThreads + t;
+        const uint32_t k = i < M ? keys[i] : 0u;
+        take[h] = k != 0 && rank_of(keys, M, k, i, i - lane) < K;
+        bal[h] = __ballot_sync(0xffffffffu, take[h]);
+        if (lane == 0) scan[h * 8 + warp] = __popc(bal[h]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if (!take[h]) continue;
+        int pos = __popc(bal[h] & ((1u << lane) - 1u));
+        for (int w = 0; w < h * 8 + warp; ++w) pos += scan[w];
+        const int m = idx[h * kScoreThreads + t];
+        lst[pos] = m;
+        if (so) so[pos] = m;
+    }
+    if (t == 0) a.list_n[bh] = K;
 }
 
 // Exact Top-K of M candidates (keys[i], block idx[i]) listed in ascending block
@@ -394,7 +441,7 @@ __global__ void __launch_bounds__(kScoreThreads) dec_score_kernel(DecodeArgs a, 
     uint4* qs = reinterpret_cast<uint4*>(smem + L.qs);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.bars);
     int* misc = reinterpret_cast<int*>(smem + L.misc);
-    uint64_t* xchg = reinterpret_cast<uint64_t*>(smem + L.xchg);
+    uint32_t* xchg = reinterpret_cast<uint32_t*>(smem + L.xchg);
     const int bh = blockIdx.y;
     const int b = bh / a.Hkv;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -403,27 +450,41 @@ __global__ void __launch_bounds__(kScoreThreads) dec_score_kernel(DecodeArgs a, 
         fence_barrier_init();
     }
     const int n = __ldg(a.seq_lens + b);
-    grid_dep_wait();     // q~ and the summary of a block closed by this step
-    grid_dep_launch();   // the attention kernel may start its set-up
-    if (bad_len(n, a)) return;   // recorded by the prep kernel
-    const int C = (n - 1) / kBlk;
+    const bool bad = bad_len(n, a);   // recorded by the prep kernel
+    const int C = bad ? 0 : (n - 1) / kBlk;
     const int K = a.topk;
     const int Kc = K > 0 ? K : 1;
     const int m0 = blockIdx.x * kDecScoreChunk;
     const int rows_cta = max(0, min(kDecScoreChunk, C - m0));
-    __syncthreads();
+    const bool scored = rows_cta > 0 && K > 0 && C > K;
+    const int r0 = m0 + warp * 32;
+    const int rows = scored ? max(0, min(32, C - r0)) : 0;
+    // the summaries, but the one of a block this step closes (the prep kernel writes
+    // it), are fetched while the prep kernel runs
+    const bool closes = rows > 0 && (n - 1) % kBlk == 0 && r0 + rows == C;
+    const bf16* ksrc = static_cast<const bf16*>(a.Ksum) + (static_cast<size_t>(bh) * a.max_blocks + r0) * DSEL;
+    const int early = rows - (closes ? 1 : 0);
+    __syncthreads();   // barriers initialised
+    if (rows > 0 && lane == 0) {
+        mbar_arrive_expect_tx(&bars[warp], static_cast<uint32_t>(rows) * kRowBytes);
+        if (early > 0)
+            bulk_load(stage + warp * kSlab, ksrc, static_cast<uint32_t>(early) * kRowBytes, &bars[warp]);
+    }
+    grid_dep_wait();     // q~ and the summary of a block closed by this step
+    grid_dep_launch();   // the attention kernel may start its set-up
+    if (bad) return;
+    if (rows > early && lane == 0)
+        bulk_load(stage + warp * kSlab + early * kRowBytes, ksrc + static_cast<size_t>(early) * DSEL, kRowBytes,
+                  &bars[warp]);
     uint32_t key = 0;
-    if (rows_cta > 0 && K > 0 && C > K) {
+    // this CTA's candidate slots: global, or (one CTA per group) its own shared
+    // memory, the ranks' key buffer once they are counted
+    const bool alone = a.nsplit_s == 1;
+    const size_t cbase = (static_cast<size_t>(bh) * a.nsplit_s + blockIdx.x) * Kc;
+    uint32_t* my_key = alone ? xchg : a.cand_key + cbase;
+    int32_t* my_idx = alone ? reinterpret_cast<int32_t*>(xchg) + Kc : a.cand_idx + cbase;
+    if (scored) {
         if (t < DSEL / 8) qs[t] = __ldg(reinterpret_cast<const uint4*>(a.qt) + static_cast<size_t>(bh) * (DSEL / 8) + t);
-        const int r0 = m0 + warp * 32;
-        const int rows = max(0, min(32, C - r0));
-        if (rows > 0 && lane == 0) {
-            const uint32_t bytes = static_cast<uint32_t>(rows) * kRowBytes;
-            mbar_arrive_expect_tx(&bars[warp], bytes);
-            bulk_load(stage + warp * kSlab,
-                      static_cast<const bf16*>(a.Ksum) + (static_cast<size_t>(bh) * a.max_blocks + r0) * DSEL, bytes,
-                      &bars[warp]);
-        }
         __syncthreads();   // q~ in shared memory
         if (rows > 0) {
             const bool ok = mbar_wait_drain(&bars[warp], 0, limit, status);
@@ -445,16 +506,12 @@ __global__ void __launch_bounds__(kScoreThreads) dec_score_kernel(DecodeArgs a, 
                 key = order_key((s0 + s1) * score_scale);
             }
         }
-        // local Top-K of this CTA's blocks: sort the distinct keys (score key, then
-        // the lower block first) and keep those at or above the K-th
+        // local Top-K of this CTA's blocks: those with fewer than K ahead of them
         bool take = t < rows_cta && key != 0;
         if (rows_cta > K) {
-            const uint64_t comp = (static_cast<uint64_t>(key) << 32) | (0xffffffffu - static_cast<uint32_t>(t));
-            const uint64_t sorted = bitonic256_desc(comp, xchg);
+            xchg[t] = take ? key : 0u;
             __syncthreads();
-            if (t == K - 1) xchg[0] = sorted;
-            __syncthreads();
-            take = take && comp >= xchg[0];
+            take = take && rank_of(xchg, (rows_cta + 3) & ~3, key, t, warp * 32) < K;
         }
         // compact the kept blocks in block order into this CTA's K candidate slots
         const unsigned bal = __ballot_sync(0xffffffffu, take);
@@ -467,35 +524,37 @@ __global__ void __launch_bounds__(kScoreThreads) dec_score_kernel(DecodeArgs a, 
             off += w < warp ? c : 0;
             total += c;
         }
-        const size_t cbase = (static_cast<size_t>(bh) * a.nsplit_s + blockIdx.x) * Kc;
         if (take) {
             const int pos = off + __popc(bal & ((1u << lane) - 1u));
-            a.cand_key[cbase + pos] = key;
-            a.cand_idx[cbase + pos] = m0 + t;
+            my_key[pos] = key;
+            my_idx[pos] = m0 + t;
         }
         for (int e = total + t; e < Kc; e += kScoreThreads) {
-            a.cand_key[cbase + e] = 0;
-            a.cand_idx[cbase + e] = -1;
+            my_key[e] = 0;
+            my_idx[e] = -1;
         }
     } else if (K > 0 && C > K) {
         // no blocks in this CTA's range: empty candidate slots
-        const size_t cbase = (static_cast<size_t>(bh) * a.nsplit_s + blockIdx.x) * Kc;
         for (int e = t; e < Kc; e += kScoreThreads) {
-            a.cand_key[cbase + e] = 0;
-            a.cand_idx[cbase + e] = -1;
+            my_key[e] = 0;
+            my_idx[e] = -1;
         }
     }
-    // the last CTA of the group to finish selects
-    __threadfence();
-    __syncthreads();
-    if (t == 0) {
-        const int old = atomicAdd(a.cnt_sel + bh, 1);
-        misc[0] = old == static_cast<int>(gridDim.x) - 1;
+    if (alone) {
+        __syncthreads();
+    } else {
+        // the last CTA of the group to finish selects
+        __threadfence();
+        __syncthreads();
+        if (t == 0) {
+            const int old = atomicAdd(a.cnt_sel + bh, 1);
+            misc[0] = old == static_cast<int>(gridDim.x) - 1;
+        }
+        __syncthreads();
+        if (!misc[0]) return;
+        __threadfence();
+        if (t == 0) a.cnt_sel[bh] = 0;   // zero again for the next launch
     }
-    __syncthreads();
-    if (!misc[0]) return;
-    __threadfence();
-    if (t == 0) a.cnt_sel[bh] = 0;   // zero again for the next launch
     int32_t* lst = a.list + static_cast<size_t>(bh) * 64;
     int32_t* so = a.sel_idx ? a.sel_idx + static_cast<size_t>(bh) * K : nullptr;
     if (C <= K) {   // short history: every historical block is kept
@@ -514,7 +573,7 @@ __global__ void __launch_bounds__(kScoreThreads) dec_score_kernel(DecodeArgs a, 
     if (C <= kDecScoreChunk) {
         // one CTA held every block: its local Top-K is the group's, already in block order
         for (int e = t; e < K; e += kScoreThreads) {
-            const int m = __ldcg(a.cand_idx + gbase + e);
+            const int m = alone ? my_idx[e] : __ldcg(a.cand_idx + gbase + e);
             lst[e] = m;
             if (so) so[e] = m;
         }
@@ -522,11 +581,17 @@ __global__ void __launch_bounds__(kScoreThreads) dec_score_kernel(DecodeArgs a, 
         return;
     }
     const int M = ((C + kDecScoreChunk - 1) / kDecScoreChunk) * Kc;   // the splits that held blocks
+    const int Mp = (M + 3) & ~3;
     uint32_t* ckeys = reinterpret_cast<uint32_t*>(stage);
-    int32_t* cidx = reinterpret_cast<int32_t*>(stage) + M;
-    for (int i = t; i < M; i += kScoreThreads) {
-        ckeys[i] = __ldcg(a.cand_key + gbase + i);
-        cidx[i] = __ldcg(a.cand_idx + gbase + i);
+    int32_t* cidx = reinterpret_cast<int32_t*>(stage) + Mp;
+    for (int i = t; i < Mp; i += kScoreThreads) {
+        ckeys[i] = i < M ? __ldcg(a.cand_key + gbase + i) : 0u;
+        cidx[i] = i < M ? __ldcg(a.cand_idx + gbase + i) : -1;
+    }
+    if (M <= kRankMax) {
+        __syncthreads();
+        select_by_rank(a, bh, M, ckeys, cidx, reinterpret_cast<int*>(smem + L.scan));
+        return;
     }
     select_candidates(a, bh, M, ckeys, cidx, reinterpret_cast<int*>(smem + L.hist),
                       reinterpret_cast<int*>(smem + L.scan), misc + 1);
@@ -863,6 +928,7 @@ constexpr int kTcThreads = 128;
 constexpr int kTcTile = 2 * 128 * 128;          // bytes of one K (or V) tile of a step
 constexpr int kTcStage = 2 * kTcTile;           // K and V
 constexpr uint32_t kTcTmemCols = 64;            // S^T in columns 0-15, O^T in 32-47
+constexpr int kMaxDecCluster = 16;              // needs the non-portable cluster size attribute
 
 struct TcLayout {
     size_t q, p, red, alpha, lsum, bars, misc, ent, total;
@@ -1013,59 +1079,64 @@ __global__ void __launch_bounds__(kTcThreads) dec_attn_tc_kernel(const __grid_co
     const uint32_t lane_base = tmem + (static_cast<uint32_t>(warp * 32) << 16);
     bool ok = true;
     int j = 0;
-    int pending = 0;   // 1: a QK commit outstanding, 2: a PV commit outstanding
+    int pending = 0, pj = 0;   // 1: a QK commit outstanding, 2: a PV commit outstanding (of step pj)
     for (; j < steps; ++j) {
         const int s = j % nst;
         uint8_t* st = smem + static_cast<size_t>(s) * kTcStage;
-        const bool got = mbar_wait_drain(&full[s], (j / nst) & 1, limit, status);
-        if (!__syncthreads_and(got)) {
-            ok = false;
-            break;
+        // Two CTA-wide barriers a step: everything else is ordered by the MMAs' commits.
+        if (warp == 0) {
+            // QK (whole warp; the elected lane issues).  Every thread has read the
+            // previous S before the barrier ahead of the previous PV.
+            ok = __all_sync(0xffffffffu, ok && mbar_wait_drain(&full[s], (j / nst) & 1, limit, status));
+            tc_fence_after();
+            if (ok && elect_one()) {
+                const uint32_t kb = smem_u32(st), qb = smem_u32(qs);
+#pragma unroll
+                for (int k = 0; k < D / 16; ++k) {
+                    const uint64_t da = smem_desc_sw128(kb + (k >> 2) * 16384 + (k & 3) * 32, 16, 1024);
+                    const uint64_t db = smem_desc_sw128(qb + (k >> 2) * 2048 + (k & 3) * 32, 16, 1024);
+                    umma_bf16(tmem, da, db, IDESC_S, k > 0);
+                }
+                umma_commit(qk_bar);
+            }
+            __syncwarp();
+            if (ok) { pending = 1; pj = j; }
         }
-        // rows of a page past its valid keys (or of a missing page) get zero values,
-        // so P = 0 there cannot meet a non-finite V
+        if (ok && !mbar_wait_drain(qk_bar, j & 1, limit, status)) ok = false;
+        ok = __all_sync(0xffffffffu, ok);
         const int e0 = 2 * j, e1 = e0 + 1;
         const int nv0 = ent[2 * e0 + 1] < 0 ? 0 : (ent[2 * e0] == c ? n - c * kBlk : kBlk);
         const int nv1 = (e1 >= cnt || ent[2 * e1 + 1] < 0) ? 0 : (ent[2 * e1] == c ? n - c * kBlk : kBlk);
-        if (nv0 < kBlk || nv1 < kBlk) {
-            for (int i = t; i < 2 * 2 * 64 * 8; i += kTcThreads) {   // (page, half, row, chunk)
-                const int pg = i >> 10, h = (i >> 9) & 1, row = (i >> 3) & 63, ch = i & 7;
-                if (row >= (pg ? nv1 : nv0))
-                    *reinterpret_cast<uint4*>(st + kTcTile + h * 16384 + pg * 8192 + row * 128 + (ch << 4)) =
-                        make_uint4(0, 0, 0, 0);
-            }
-            fence_proxy_async_smem();
-            __syncthreads();
-        }
-        if (t == 0) {
-            tc_fence_after();
-            const uint32_t kb = smem_u32(st), qb = smem_u32(qs);
-#pragma unroll
-            for (int k = 0; k < D / 16; ++k) {
-                const uint64_t da = smem_desc_sw128(kb + (k >> 2) * 16384 + (k & 3) * 32, 16, 1024);
-                const uint64_t db = smem_desc_sw128(qb + (k >> 2) * 2048 + (k & 3) * 32, 16, 1024);
-                umma_bf16(tmem, da, db, IDESC_S, k > 0);
-            }
-            umma_commit(qk_bar);
-        }
-        pending = 1;
-        if (!mbar_wait_drain(qk_bar, j & 1, limit, status)) ok = false;
-        if (!__syncthreads_and(ok)) break;
-        pending = 0;
         tc_fence_after();
-        uint32_t sr[16];
-        tmem_ld16(lane_base, sr);
-        tmem_wait_ld();
         const int key = t;                           // TMEM lane = key of the pair
         const bool valid = key < 64 ? key < nv0 : key - 64 < nv1;
         float z[G];
+        if (ok) {
+            uint32_t sr[16];
+            tmem_ld16(lane_base, sr);
+            tmem_wait_ld();
 #pragma unroll
-        for (int h = 0; h < G; ++h) {
-            z[h] = valid ? __uint_as_float(sr[h]) * scale_log2 : -CUDART_INF_F;
-            const float mx = warp_max(z[h]);
-            if (lane == 0) red[warp * 16 + h] = mx;
+            for (int h = 0; h < G; ++h) {
+                z[h] = valid ? __uint_as_float(sr[h]) * scale_log2 : -CUDART_INF_F;
+                const float mx = warp_max(z[h]);
+                if (lane == 0) red[warp * 16 + h] = mx;
+            }
+            // rows of a page past its valid keys (or of a missing page) get zero values,
+            // so P = 0 there cannot meet a non-finite V
+            if (nv0 < kBlk || nv1 < kBlk) {
+                mbar_wait_drain(&full[s], (j / nst) & 1, limit, status);   // completed: QK has read the stage
+                for (int i = t; i < 2 * 2 * 64 * 8; i += kTcThreads) {   // (page, half, row, chunk)
+                    const int pg = i >> 10, h = (i >> 9) & 1, row = (i >> 3) & 63, ch = i & 7;
+                    if (row >= (pg ? nv1 : nv0))
+                        *reinterpret_cast<uint4*>(st + kTcTile + h * 16384 + pg * 8192 + row * 128 + (ch << 4)) =
+                            make_uint4(0, 0, 0, 0);
+                }
+            }
         }
-        __syncthreads();
+        if (!__syncthreads_and(ok)) {
+            ok = false;
+            break;
+        }
         float alpha[G];
 #pragma unroll
         for (int h = 0; h < G; ++h) {
@@ -1082,30 +1153,36 @@ __global__ void __launch_bounds__(kTcThreads) dec_attn_tc_kernel(const __grid_co
         fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();
-        if (t == 0) {
+        if (warp == 0) {
             tc_fence_after();
-            const uint32_t vb = smem_u32(st + kTcTile), pb = smem_u32(ps);
+            if (elect_one()) {
+                const uint32_t vb = smem_u32(st + kTcTile), pb = smem_u32(ps);
 #pragma unroll
-            for (int k = 0; k < 128 / 16; ++k) {
-                const uint64_t da = smem_desc_sw128(vb + k * 2048, 16384, 1024);
-                const uint64_t db = smem_desc_sw128(pb + (k >> 2) * 2048 + (k & 3) * 32, 16, 1024);
-                umma_bf16(tmem + 32, da, db, IDESC_O, k > 0);
+                for (int k = 0; k < 128 / 16; ++k) {
+                    const uint64_t da = smem_desc_sw128(vb + k * 2048, 16384, 1024);
+                    const uint64_t db = smem_desc_sw128(pb + (k >> 2) * 2048 + (k & 3) * 32, 16, 1024);
+                    umma_bf16(tmem + 32, da, db, IDESC_O, k > 0);
+                }
+                umma_commit(pv_bar);
             }
-            umma_commit(pv_bar);
+            __syncwarp();
+            pending = 2;
         }
-        pending = 2;
         if (!mbar_wait_drain(pv_bar, j & 1, limit, status)) ok = false;
-        if (!__syncthreads_and(ok)) break;
-        pending = 0;
-        tc_fence_after();
-        uint32_t orr[16];
-        tmem_ld16(lane_base + 32, orr);
-        tmem_wait_ld();
+        ok = __all_sync(0xffffffffu, ok);
+        if (ok) {
+            pending = 0;
+            tc_fence_after();
+            uint32_t orr[16];
+            tmem_ld16(lane_base + 32, orr);
+            tmem_wait_ld();
 #pragma unroll
-        for (int h = 0; h < G; ++h) o[h] = fmaf(o[h], alpha[h], __uint_as_float(orr[h]));
-        tc_fence_before();
-        __syncthreads();   // the stage, P and the TMEM columns are free
-        if (t == 0 && issued < steps) {
+            for (int h = 0; h < G; ++h) o[h] = fmaf(o[h], alpha[h], __uint_as_float(orr[h]));
+            tc_fence_before();
+        }
+        // (a warp that gave up here says so at the next step's barrier)
+        // PV has read the stage: its next load can go out
+        if (t == 0 && ok && issued < steps) {
             const int e0 = 2 * issued, e1 = e0 + 1;
             const int s2 = issued % nst;
             uint32_t bytes = tc_page_bytes(ent, e0);
@@ -1116,12 +1193,12 @@ __global__ void __launch_bounds__(kTcThreads) dec_attn_tc_kernel(const __grid_co
             ++issued;
         }
     }
-    if (!ok) {
+    if (!__syncthreads_and(ok)) {
         // let the tensor cores and the copies in flight finish before leaving
         if (t == 0) {
-            if (pending == 1) mbar_wait_drain(qk_bar, j & 1, limit, status);
-            if (pending == 2) mbar_wait_drain(pv_bar, j & 1, limit, status);
-            for (int q = j; q < issued; ++q) mbar_wait_drain(&full[q % nst], (q / nst) & 1, limit, status);
+            if (pending == 1) mbar_wait_drain(qk_bar, pj & 1, limit, status);
+            if (pending == 2) mbar_wait_drain(pv_bar, pj & 1, limit, status);
+            for (int q = max(0, issued - nst); q < issued; ++q) mbar_wait_drain(&full[q % nst], (q / nst) & 1, limit, status);
         }
 #pragma unroll
         for (int h = 0; h < G; ++h) {
@@ -1144,6 +1221,45 @@ __global__ void __launch_bounds__(kTcThreads) dec_attn_tc_kernel(const __grid_co
         if (lane == 0) lsum[warp * 16 + h] = ls;
     }
     __syncthreads();
+    if (a.cluster) {
+        // the group's CTAs are one cluster: each leaves its partials in its shared
+        // memory (the free stage) and merges the heads h = rank, rank + S, ...
+        float* mine = reinterpret_cast<float*>(smem);   // [G][D + 2]
+#pragma unroll
+        for (int h = 0; h < G; ++h) {
+            if (t == 0) {
+                mine[h * (D + 2)] = m_run[h];
+                mine[h * (D + 2) + 1] = lsum[h] + lsum[16 + h] + lsum[32 + h] + lsum[48 + h];
+            }
+            mine[h * (D + 2) + 2 + t] = o[h];
+        }
+        cluster_sync();
+        const int S = cluster_size();
+        const uint32_t own = smem_u32(mine);
+        for (int h = cluster_rank(); h < G && !bad; h += S) {
+            const uint32_t at = own + h * (D + 2) * 4;
+            float mx[kMaxDecCluster], M = -CUDART_INF_F;
+#pragma unroll
+            for (int x = 0; x < kMaxDecCluster; ++x) {
+                mx[x] = x < S ? dsmem_ld_f(cluster_map(at, x)) : -CUDART_INF_F;
+                M = fmaxf(M, mx[x]);
+            }
+            float ls = 0.f, acc = 0.f;
+#pragma unroll
+            for (int x = 0; x < kMaxDecCluster; ++x) {
+                if (x >= S) break;
+                const float w = mx[x] == -CUDART_INF_F ? 0.f : fast_exp2(mx[x] - M);
+                ls = fmaf(w, dsmem_ld_f(cluster_map(at + 4, x)), ls);
+                acc = fmaf(w, dsmem_ld_f(cluster_map(at + 8 + t * 4, x)), acc);
+            }
+            const size_t orow = (static_cast<size_t>(b) * a.Hq + static_cast<size_t>(g) * G + h) * D;
+            static_cast<bf16*>(a.O)[orow + t] = __float2bfloat16_rn(acc / ls);
+            if (a.LSE != nullptr && t == 0)
+                a.LSE[static_cast<size_t>(b) * a.Hq + static_cast<size_t>(g) * G + h] = (M + log2f(ls)) / kLog2e;
+        }
+        cluster_sync();   // the peers have read this CTA's partials
+        return;
+    }
     float* part = a.part + (static_cast<size_t>(bh) * a.nsplit_a + blockIdx.x) * G * (D + 2);
 #pragma unroll
     for (int h = 0; h < G; ++h) {
@@ -1205,19 +1321,24 @@ __global__ void __launch_bounds__(kTcThreads) dec_attn_tc_kernel(const __grid_co
 
 // Launch with programmatic stream serialization: the kernel may start while
 // the preceding kernel on the stream still runs (it waits with griddepcontrol).
+// cluster > 1: the CTAs of a grid row form clusters of that many.
 template <class... KArgs, class... Args>
-cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                             Args... args) {
+cudaError_t launch_dependent(int cluster, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                             cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -1235,14 +1356,14 @@ cudaError_t launch_attn_dg(const DecodeArgs& a, const KernelEnv& env) {
     cudaError_t e = prepare_attn_dg<D, G>(a);
     if (e != cudaSuccess) return e;
     dim3 grid(a.nsplit_a, a.B * a.Hkv);
-    return launch_dependent(dec_attn_kernel<D, G>, grid, dim3(kAttnThreads), smem, env.stream, a, env.status,
+    return launch_dependent(1, dec_attn_kernel<D, G>, grid, dim3(kAttnThreads), smem, env.stream, a, env.status,
                             env.limit, a.sm_scale * kLog2e);
 }
 
 template <int G>
 cudaError_t prepare_attn_tc(const DecodeArgs& a) {
     const size_t smem = tc_layout(a.nst, a.bpc).total;
-    return ensure_smem_attr(reinterpret_cast<const void*>(dec_attn_tc_kernel<G>), smem);
+    return ensure_smem_attr(reinterpret_cast<const void*>(dec_attn_tc_kernel<G>), smem, false, true);
 }
 
 template <int G>
@@ -1254,7 +1375,7 @@ cudaError_t launch_attn_tc(const DecodeArgs& a, const KernelEnv& env) {
     if (make_tmap_bf16_3d(&mk, a.K_cache, 128, kBlk, rows, 64, kBlk) != 0) return cudaErrorInvalidValue;
     if (make_tmap_bf16_3d(&mv, a.V_cache, 128, kBlk, rows, 64, kBlk) != 0) return cudaErrorInvalidValue;
     dim3 grid(a.nsplit_a, a.B * a.Hkv);
-    return launch_dependent(dec_attn_tc_kernel<G>, grid, dim3(kTcThreads), tc_layout(a.nst, a.bpc).total, env.stream,
+    return launch_dependent(a.cluster ? a.nsplit_a : 1, dec_attn_tc_kernel<G>, grid, dim3(kTcThreads), tc_layout(a.nst, a.bpc).total, env.stream,
                             mk, mv, a, env.status, env.limit, a.sm_scale * kLog2e);
 }
 
@@ -1310,18 +1431,35 @@ cudaError_t launch_score_d(const DecodeArgs& a, const KernelEnv& env) {
     cudaError_t e = prepare_score_d<DSEL>(a);
     if (e != cudaSuccess) return e;
     dim3 grid(a.nsplit_s, a.B * a.Hkv);
-    return launch_dependent(dec_score_kernel<DSEL>, grid, dim3(kScoreThreads), smem, env.stream, a, env.status,
+    return launch_dependent(1, dec_score_kernel<DSEL>, grid, dim3(kScoreThreads), smem, env.stream, a, env.status,
                             env.limit, static_cast<float>(1.0 / sqrt(static_cast<double>(DSEL))));
 }
 
 }  // namespace
 
-void decode_attn_split(int max_len, int d, int* nsplit, int* bpc, int* nst) {
+void decode_attn_split(int max_len, int d, bool dense, int groups, int sms, int* nsplit, int* bpc, int* nst,
+                       int* cluster) {
     int per;
-    if (d == 128) {
-        // tensor-core kernel: two pages (one 128-key step) per CTA for a SAS list;
-        // long dense lists cut into at most 64 (128 past 2048 pages) pieces of
-        // whole steps.  One stage, so that three CTAs share an SM and overlap one
+    *cluster = 0;
+    if (d == 128 && !dense) {
+        // tensor-core kernel, a SAS list (at most 65 pages): a cluster of S <= 16 CTAs
+        // per group, as many as run at once, merging over distributed shared memory.
+        // Three CTAs of one 64 KB stage share an SM, but whole clusters have to find
+        // room in a GPC, so the grid stays at 8/3 of the SMs (64 groups of 33 pages:
+        // 28.8, 25.7, 23.6, 20.8 and 32.0 us with S = 3, 4, 5, 6 and 7).  One CTA per
+        // SM or fewer: up to three stages, so that a CTA's own loads overlap.  (Before:
+        // one page pair per CTA and a merge through global memory by the last one to
+        // arrive; 64 groups took 2.4 waves and 36.5 us.)
+        const int fit = 8 * sms / (3 * (groups > 0 ? groups : 1));
+        int S = fit < 1 ? 1 : (fit > kMaxDecCluster ? kMaxDecCluster : fit);
+        per = (max_len + S - 1) / S;
+        S = (max_len + per - 1) / per;
+        const int steps = (per + 1) / 2;
+        *nst = static_cast<long long>(groups) * S <= sms ? (steps < 3 ? steps : 3) : 1;
+        *cluster = 1;
+    } else if (d == 128) {
+        // dense lists: cut into at most 64 (128 past 2048 pages) pieces of whole
+        // steps.  One stage, so that three CTAs share an SM and overlap one
         // another's loads (two stages and one CTA per SM measured slower).
         const int pieces = max_len <= 2048 ? 64 : 128;   // long lists: more CTAs pay for the larger merge
         per = max_len <= 96 ? 2 : 2 * ((max_len + 2 * pieces - 1) / (2 * pieces));

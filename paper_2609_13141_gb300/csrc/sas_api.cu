@@ -56,7 +56,7 @@ std::map<std::pair<const void*, int>, size_t> g_smem_attr;   // (kernel, device)
 std::map<int, int> g_sms;                                     // device -> SM count
 }  // namespace
 
-cudaError_t ensure_smem_attr(const void* func, size_t bytes, bool max_carveout) {
+cudaError_t ensure_smem_attr(const void* func, size_t bytes, bool max_carveout, bool big_clusters) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -66,6 +66,8 @@ cudaError_t ensure_smem_attr(const void* func, size_t bytes, bool max_carveout) 
     e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
     if (e == cudaSuccess && max_carveout)
         e = cudaFuncSetAttribute(func, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess && big_clusters)
+        e = cudaFuncSetAttribute(func, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) set = bytes;
     return e;
 }

@@ -23,7 +23,7 @@ struct sas_decode_handle {
     sas_decode_config cfg;
     int G = 1, d_sel = 0;
     float sm_scale = 0.f;
-    int nsplit_s = 0, nsplit_a = 0, bpc = 0, nst = 0;
+    int nsplit_s = 0, nsplit_a = 0, bpc = 0, nst = 0, cluster = 0;
     // workspace
     void* qt = nullptr;
     uint32_t* cand_key = nullptr;
@@ -104,7 +104,7 @@ sas::DecodeArgs base_args(const sas_decode_handle* h) {
     a.qt = h->qt; a.cand_key = h->cand_key; a.cand_idx = h->cand_idx; a.list = h->list; a.list_n = h->list_n; a.part = h->part;
     a.cnt_sel = h->counters;
     a.cnt_attn = h->counters + static_cast<size_t>(c.B) * c.Hkv;
-    a.nsplit_s = h->nsplit_s; a.nsplit_a = h->nsplit_a; a.bpc = h->bpc; a.nst = h->nst;
+    a.nsplit_s = h->nsplit_s; a.nsplit_a = h->nsplit_a; a.bpc = h->bpc; a.nst = h->nst; a.cluster = h->cluster;
     return a;
 }
 
@@ -138,7 +138,8 @@ sas_status sas_decode_create(const sas_decode_config* cfg, sas_decode_handle** o
     h->d_sel = d_sel;
     h->sm_scale = c.sm_scale > 0.f ? c.sm_scale : 1.0f / std::sqrt(static_cast<float>(c.d));
     h->nsplit_s = (c.max_blocks + sas::kDecScoreChunk - 1) / sas::kDecScoreChunk;
-    sas::decode_attn_split(c.dense ? c.max_blocks : c.topk + 1, c.d, &h->nsplit_a, &h->bpc, &h->nst);
+    sas::decode_attn_split(c.dense ? c.max_blocks : c.topk + 1, c.d, c.dense != 0, static_cast<int>(BH),
+                           sas::device_sm_count(), &h->nsplit_a, &h->bpc, &h->nst, &h->cluster);
 
     int dev = 0, major = 0, minor = 0;
     cudaError_t e = cudaGetDevice(&dev);
