@@ -216,6 +216,7 @@ struct AttnBwdArgs {
     int32_t* inv_pos;           // their block positions
     int32_t* slot_off;          // [BH*T + 1] first offset slot of each tile
     float* offs;                // [slots][128] per-row offsets written by pass 1
+    uint8_t* live;              // [slots][4] whether each quarter of the rows attends the block
     // packed sequences: the forward's tile table (as in SelectArgs) and its
     // per-local-tile first slots; null for [B, H, N, d] batches
     const int4* tiles;

@@ -16,7 +16,11 @@
 //   bwd_dkv_kernel    pass 2, one CTA per (head, key pair) over those query
 //                     tiles, 64 rows at a time: S^T = K Q^T, dP^T = V dO^T
 //                     into two TMEM buffers, P^T and dS^T written in place
-//                     over them, dV += P^T dO and dK += dS^T Q.
+//                     over them, dV += P^T dO and dK += dS^T Q.  Bound by the
+//                     latency of a half's loads and hand-offs (1.13 ms at 24
+//                     heads x 16896 tokens, K = 32, block-coherent scores; 1.75
+//                     before halves were loaded one by one and those no row of
+//                     which attends the pair left out, a third of them there).
 //   bwd_ds_kernel     score gradient of given scores (sparse scope):
 //                     ds_m = dlogg_m [m kept] - g_m sum dlogg.
 //   bwd_dense_*       kept lists and tile unions of every historical block:
@@ -125,6 +129,7 @@ struct BwdParams {
     const int32_t* inv_pos;     // per inverted entry: positions of blocks 2p, 2p+1 in the tile's list (+1; 0: absent)
     const int32_t* slot_off;    // per tile: first slot of its visited blocks in offs
     float* offs;                // per (tile, visited block) slot: 128 rows of log g - LSE (log2), -inf if not attended
+    uint8_t* live;              // per slot: whether rows 32 w .. 32 w + 31 attend the block at all, w = 0 .. 3
     const int4* tiles;          // packed sequences: {first row of the sequence, local tile, length, sequence} per slot
     const int* ntiles;          // slots in use (device)
     const int* tile_off;        // first slot of each local tile index
@@ -404,6 +409,9 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ 
                 const float boff = lim >= 0 ? (OUTER ? -lse2 : bias - lse2) : -CUDART_INF_F;
                 const float wg = OUTER ? fast_exp2(bias) : 1.f;
                 const bool causal = lim >= 0 && lim < kKeys - 1;
+                const bool some = __any_sync(0xffffffffu, lim >= 0);
+                if (hk == 0 && lane == 0 && p.offs != nullptr)
+                    p.live[(static_cast<long long>(slot0) + j) * 4 + warp] = some ? 1 : 0;
                 if (hk == 0 && p.offs != nullptr)
                     p.offs[(static_cast<long long>(slot0) + j) * kRows + r] = OUTER ? (lim >= 0 ? wg : -1.f) : boff;
                 const uint64_t sc2 = f32x2(p.scale_log2, p.scale_log2), bo2 = f32x2(boff, boff);
@@ -503,11 +511,15 @@ __device__ __forceinline__ InvSrc inv_src(int g, int hg, const int4* tiles, cons
 
 // count: for every tile (head-packed: segment), the key pairs (2p, 2p+1) its
 // union list touches, but its own pair; nsrc tiles or segments per group,
-// union rows of ustride; hg = G for head-packed segments, else 0
-__global__ void bwd_inv_count_kernel(const int32_t* union_idx, const int32_t* union_cnt, int32_t* cnt, int BH,
-                                     int T, int nsrc, int ustride, const int4* tiles, const int* ntiles,
-                                     const int* tile_off, int hg) {
-    const long long tb = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+// union rows of ustride; hg = G for head-packed segments, else 0.  A warp per
+// source, a lane per list entry (a thread per source walked its list alone: 67
+// us for count and fill at 24 heads x 16896 tokens, K = 32)
+__global__ void __launch_bounds__(256) bwd_inv_count_kernel(const int32_t* union_idx, const int32_t* union_cnt,
+                                                            int32_t* cnt, int BH, int T, int nsrc, int ustride,
+                                                            const int4* tiles, const int* ntiles, const int* tile_off,
+                                                            int hg) {
+    const long long tb = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (tb >= static_cast<long long>(BH) * nsrc) return;
     const int bh = static_cast<int>(tb / nsrc);
     const int g = static_cast<int>(tb - static_cast<long long>(bh) * nsrc);
@@ -515,11 +527,10 @@ __global__ void bwd_inv_count_kernel(const int32_t* union_idx, const int32_t* un
     if (src.ts < 0) return;
     const int32_t* u = union_idx + tb * ustride;
     const int U = union_cnt[tb];
-    int last = -1;
-    for (int k = 0; k < U; ++k) {
+    for (int k = lane; k < U; k += 32) {
         const int pr = u[k] >> 1;
-        if (pr == last || pr == src.own) continue;
-        last = pr;
+        // the list ascends: the pair's first entry counts it
+        if ((k > 0 && (u[k - 1] >> 1) == pr) || pr == src.own) continue;
         atomicAdd(cnt + static_cast<long long>(bh) * T + pair_slot(tiles, tile_off, src.ts, pr), 1);
     }
 }
@@ -552,10 +563,12 @@ __global__ void __launch_bounds__(1024) bwd_inv_scan_kernel(const int32_t* cnt, 
 
 // fill: entry = the visiting tile's index within its sequence (head-packed: the
 // segment's) and the positions of the pair's blocks in its list
-__global__ void bwd_inv_fill_kernel(const int32_t* union_idx, const int32_t* union_cnt, int32_t* cursor,
-                                    int32_t* tiles, int32_t* pos, int BH, int T, int nsrc, int ustride,
-                                    const int4* ttab, const int* ntiles, const int* tile_off, int hg) {
-    const long long tb = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(256) bwd_inv_fill_kernel(const int32_t* union_idx, const int32_t* union_cnt,
+                                                           int32_t* cursor, int32_t* tiles, int32_t* pos, int BH,
+                                                           int T, int nsrc, int ustride, const int4* ttab,
+                                                           const int* ntiles, const int* tile_off, int hg) {
+    const long long tb = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (tb >= static_cast<long long>(BH) * nsrc) return;
     const int bh = static_cast<int>(tb / nsrc);
     const int g = static_cast<int>(tb - static_cast<long long>(bh) * nsrc);
@@ -563,11 +576,9 @@ __global__ void bwd_inv_fill_kernel(const int32_t* union_idx, const int32_t* uni
     if (src.ts < 0) return;
     const int32_t* u = union_idx + tb * ustride;
     const int U = union_cnt[tb];
-    int last = -1;
-    for (int k = 0; k < U; ++k) {
+    for (int k = lane; k < U; k += 32) {
         const int m = u[k], pr = m >> 1;
-        if (pr == last || pr == src.own) continue;
-        last = pr;
+        if ((k > 0 && (u[k - 1] >> 1) == pr) || pr == src.own) continue;
         // positions (+1) of blocks 2pr and 2pr+1 in this tile's list (ascending)
         const int j0 = m == 2 * pr ? k + 1 : 0;
         const int j1 = m == 2 * pr + 1 ? k + 1 : (k + 1 < U && u[k + 1] == 2 * pr + 1 ? k + 2 : 0);
@@ -631,24 +642,31 @@ __global__ void bwd_dlogg_sum_kernel(const float* heads, float* out, long long p
 // ------------------------------------------------------------------ pass 2
 
 struct DkvCtl {
-    uint64_t kv_full, q_full[2], q_empty[2], info_full[4], info_empty[4];
+    uint64_t kv_full, q_full[4], q_empty[4], info_full[4], info_empty[4];
     uint64_t sdp_full[2], pds_full[2], fin;   // per TMEM buffer
     uint32_t tmem_base;
     int abort_flag;
+    int nh;                                   // 64-row halves to process
 };
 
 constexpr int kThreadsD = 256;                           // keys (4 warps), two issuers, a row-info warp, a loader
 constexpr int kInfoLanes = 32;
 constexpr int kPairBytes = 2 * kKeys * kD * 2;           // 32 KB: K (or V) of the key pair
 constexpr int kDkvOffV = kPairBytes;
-constexpr int kDkvOffQ = 2 * kPairBytes;                 // 2 stages x (Q, dO) tiles
+constexpr int kDkvOffQ = 2 * kPairBytes;                 // kQStages x (Q, dO) of 64 rows
+// Q and dO rows come by halves of an item: a half's products start when its own 32
+// KB are in, three more halves are in flight behind it, and a half left out is not
+// loaded.  (As two stages of whole 128-row tiles, items of one half waited for
+// their loads: leaving a third of the halves out gained 3%.)
+constexpr int kQStages = 4;
+constexpr int kQHalfBytes = kQBytes / 2;                 // 64 rows of Q (or dO)
 constexpr int kInfoStages = 4;                           // row information computed up to 3 tiles ahead
-constexpr int kDkvOffInfo = kDkvOffQ + 2 * 2 * kQBytes;  // stages x [4][128] floats: lse2, delta, bias0, bias1
+constexpr int kDkvOffInfo = kDkvOffQ + kQStages * 2 * kQHalfBytes;  // stages x [4][128] floats: lse2, delta, bias0, bias1
 constexpr int kDkvOffList = kDkvOffInfo + kInfoStages * 4 * kRows * 4;
 // query tiles of a key pair (sorted list, then the unsorted copy); the host
 // refuses heads of more than kBwdMaxTiles tiles
 constexpr int kDkvListCap = 2048;
-constexpr int kDkvOffCtl = kDkvOffList + 3 * kDkvListCap * 4;   // order, tiles, positions
+constexpr int kDkvOffCtl = kDkvOffList + 3 * kDkvListCap * 4;   // halves (16 bits, two a tile), tiles, positions
 constexpr int kDkvSmem = kDkvOffCtl + 256 + 1024;
 // TMEM: dV [0,128), dK [128,256), then two buffers b of 128 columns at 256 + 128 b:
 // S^T in the first 64, dP^T in the last 64.  The keys write P^T (dS^T) in place
@@ -662,7 +680,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     extern __shared__ __align__(1024) uint8_t dsm[];
     uint8_t* smem = dsm + ((1024u - (smem_u32(dsm) & 1023u)) & 1023u);
     DkvCtl& ctl = *reinterpret_cast<DkvCtl*>(smem + kDkvOffCtl);
-    int* list = reinterpret_cast<int*>(smem + kDkvOffList);
+    uint16_t* hl = reinterpret_cast<uint16_t*>(smem + kDkvOffList);   // see half_at
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     // key pair = blocks 2pr, 2pr+1 (keys 128 pr .. of the sequence) of group kv; its
     // slot is that of the sequence's local tile pr
@@ -686,9 +704,9 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     const int nitems = nq * G;
     if (t == 0) {
         mbar_init(&ctl.kv_full, 1);
-        for (int s = 0; s < 2; ++s) {
+        for (int s = 0; s < kQStages; ++s) {
             mbar_init(&ctl.q_full[s], 1);
-            mbar_init(&ctl.q_empty[s], 2);    // both issuers' products of the tile
+            mbar_init(&ctl.q_empty[s], 2);    // both issuers' accumulations of the half
         }
         for (int s = 0; s < kInfoStages; ++s) {
             mbar_init(&ctl.info_full[s], 1);                // the row-information warp
@@ -708,18 +726,41 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     }
     // the query tiles: diagonal first, then the others in ascending order (a
     // fixed summation order); rank sort of the inverted list in shared memory
-    // list[q]: index into raw / rawpos of the q-th query tile (slot 0: the diagonal
-    // tile, which visits 2pr, 2pr+1 right after its union list); raw holds the
-    // tiles' indices within the sequence (so packed sequences sum in the order of
-    // a batch of the same data)
-    int* raw = list + kDkvListCap;
+    // slot 0 of raw / rawpos: the diagonal tile, which visits 2pr, 2pr+1 right
+    // after its union list; raw holds the tiles' indices within the sequence (so
+    // packed sequences sum in the order of a batch of the same data).
+    // hl: the 64-row halves to process, in that order: index into raw << 3 |
+    // first of its item << 1 | last of its item << 2 | half.  Per-head tiles
+    // leave out the halves no row of which attends either block (pass 1's
+    // `live` bytes): where a query block's rows keep the same blocks, about half
+    // of them beyond the short histories.
+    int* raw = reinterpret_cast<int*>(smem + kDkvOffList) + kDkvListCap;
     int* rawpos = raw + kDkvListCap;
+    const bool skip = !hp && G == 1;
+    // halves of per-head tile index tq with block positions ps that some row attends
+    auto halves = [&](int tq, int ps) -> int {
+        if (!skip) return 3;
+        int gq = tq;
+        if (p.tiles != nullptr) gq = pslot - __ldg(p.tile_off + pr) + __ldg(p.tile_off + tq);
+        const long long so = __ldg(p.slot_off + static_cast<long long>(kv) * p.T + gq);
+        const int j0 = (ps & 0xffff) - 1, j1 = (ps >> 16) - 1;
+        uint32_t w = 0;
+        if (j0 >= 0) w |= __ldcg(reinterpret_cast<const uint32_t*>(p.live) + so + j0);
+        if (j1 >= 0) w |= __ldcg(reinterpret_cast<const uint32_t*>(p.live) + so + j1);
+        return ((w & 0xffffu) != 0 ? 1 : 0) | ((w >> 16) != 0 ? 2 : 0);
+    };
+    auto put_halves = [&](int pos, int r, int hm) {
+        if (hm & 1) hl[pos++] = static_cast<uint16_t>(r << 3 | (hm & 2 ? 0 : 4) | 2);
+        if (hm & 2) hl[pos] = static_cast<uint16_t>(r << 3 | 4 | (hm & 1 ? 0 : 2) | 1);
+    };
     if (t == 0) {
         if (!hp) {
-            list[0] = 0;
             raw[0] = pr;
             const int Upr = __ldg(p.union_cnt + pb);
-            rawpos[0] = (Upr + 1) | ((2 * pr + 1 < cseq ? Upr + 2 : 0) << 16);
+            const int ps = (Upr + 1) | ((2 * pr + 1 < cseq ? Upr + 2 : 0) << 16);
+            const int hm = halves(pr, ps);
+            rawpos[0] = ps | (hm & 1 ? 1 << 15 : 0) | (hm & 2 ? 1 << 31 : 0);
+            put_halves(0, 0, hm);
         } else {
             // segment sg of block c visits c right after its union (position U); a
             // segment of block 2 pr + 1 may also keep block 2 pr (its union's last entry)
@@ -735,22 +776,28 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
                     const bool has0 = Us > 0 && __ldg(p.seg_union_idx + sb * p.seg_cap + Us - 1) == 2 * pr;
                     pos = (has0 ? Us : 0) | ((Us + 1) << 16);
                 }
-                list[k] = k;
                 raw[k] = sg;
-                rawpos[k] = pos;
+                rawpos[k] = pos | 1 << 15 | 1 << 31;
+                put_halves(2 * k, k, 3);
             }
         }
     }
     for (int k = t; k < cnt; k += kThreadsD) {
-        raw[ndg + k] = __ldg(p.inv_tiles + off + k);
-        rawpos[ndg + k] = __ldg(p.inv_pos + off + k);
+        const int tq = __ldg(p.inv_tiles + off + k), ps = __ldg(p.inv_pos + off + k);
+        const int hm = halves(tq, ps);
+        raw[ndg + k] = tq;
+        rawpos[ndg + k] = ps | (hm & 1 ? 1 << 15 : 0) | (hm & 2 ? 1 << 31 : 0);
     }
     __syncthreads();
+    const int dh = hp ? 2 * ndg : __popc(rawpos[0] & 0x80008000);   // halves of the diagonal item(s)
+    if (t == 0) ctl.nh = dh;
+    __syncthreads();
     for (int k = t; k < cnt; k += kThreadsD) {
-        const int v = raw[ndg + k];
-        int rank = 0;
-        for (int q = 0; q < cnt; ++q) rank += raw[ndg + q] < v;
-        list[ndg + rank] = ndg + k;
+        const int v = raw[ndg + k], hb = rawpos[ndg + k] & 0x80008000;
+        int before = 0;
+        for (int q = 0; q < cnt; ++q) before += raw[ndg + q] < v ? __popc(rawpos[ndg + q] & 0x80008000) : 0;
+        put_halves(dh + before, ndg + k, (hb & 0x8000 ? 1 : 0) | (hb < 0 ? 2 : 0));
+        atomicAdd(&ctl.nh, __popc(hb));
     }
     tc_fence_before();
     __syncthreads();
@@ -758,28 +805,50 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
     const uint32_t tmem = ctl.tmem_base;
     const WaitCtl wc{&ctl.abort_flag, p.status, p.limit};
     float* info = reinterpret_cast<float*>(smem + kDkvOffInfo);
-    const int nh = 2 * nitems;   // 64-row halves of the items
+    // 64-row halves of the items; half x: index into raw, query head of the group,
+    // half, whether it is its item's first / last
+    const int nh = skip ? ctl.nh : 2 * nitems;
+    auto half_at = [&](int x, int& r, int& head, int& h, bool& first, bool& last) {
+        if (skip) {
+            const int v = hl[x];
+            r = v >> 3;
+            head = 0;
+            h = v & 1;
+            first = (v & 2) != 0;
+            last = (v & 4) != 0;
+        } else {
+            r = hl[2 * ((x >> 1) / G)] >> 3;
+            head = (x >> 1) % G;
+            h = x & 1;
+            first = h == 0;
+            last = h == 1;
+        }
+    };
 
     if (warp == 5) {
         // ---- row information of query tile q, up to three tiles ahead: per row
         // the offsets (log g - LSE) of blocks 2pr, 2pr+1 that pass 1 wrote, and -Delta
         const int il = lane;
-        for (int it = 0; it < nitems; ++it) {
+        int it = 0;   // items so far
+        for (int x = 0; x < nh; ++x) {
+            int ri, head, hx;
+            bool fst, lst;
+            half_at(x, ri, head, hx, fst, lst);
+            if (!fst) continue;
             const int s = it % kInfoStages;
             if (it >= kInfoStages &&
                 !mbar_wait(&ctl.info_empty[s], ((it - kInfoStages) / kInfoStages) & 1, wc, kSleepNs))
                 break;
             float* inf = info + s * 4 * kRows;
-            const int q = it / G;
-            const int bhq = kv * G + it % G;   // the item's query head (per-head tiles)
-            const int tq = raw[list[q]];       // the query tile within the sequence (head-packed: segment), and its slot
+            const int bhq = kv * G + head;     // the item's query head (per-head tiles)
+            const int tq = raw[ri];            // the query tile within the sequence (head-packed: segment), and its slot
             int gq = tq;
             if (p.tiles != nullptr) {
                 const int tt = hp ? tq / p.G : tq;   // the local tile
                 gq = pslot - __ldg(p.tile_off + pr) + __ldg(p.tile_off + tt);
                 if (hp) gq = gq * p.G + (tq - tt * p.G);
             }
-            const int ps = rawpos[list[q]];
+            const int ps = rawpos[ri] & 0x7fff7fff;
             const int j0 = (ps & 0xffff) - 1, j1 = (ps >> 16) - 1;
             const long long tbq = hp ? static_cast<long long>(kv) * p.nseg + gq : static_cast<long long>(bhq) * p.T + gq;
             const long long so = static_cast<long long>(__ldg(p.slot_off + tbq)) * kRows;
@@ -798,38 +867,36 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
                 if (OUTER) inf[3 * kRows + r] = i < ptg.n ? -__ldg(p.LSE + drow) * kLog2eB : -CUDART_INF_F;
             }
             mbar_arrive_warp(&ctl.info_full[s]);
+            ++it;
         }
     } else if (warp == 6) {
         if (lane == 0) {
             // ---- loader: K and V of the pair once, then the (Q, dO) rows of
-            // query tile q into stage q & 1 once both products of tile q - 2 are done
+            // half x into stage x % kQStages once both accumulations of half x - kQStages are done
             mbar_arrive_expect_tx(&ctl.kv_full, 2 * kPairBytes);
             for (int h = 0; h < 2; ++h) {
                 tma_load_3d(smem + h * (2 * kKeys * 128), &mapK2, &ctl.kv_full, h * 64, ptg.base + pr * 2 * kKeys, kv);
                 tma_load_3d(smem + kDkvOffV + h * (2 * kKeys * 128), &mapV2, &ctl.kv_full, h * 64,
                             ptg.base + pr * 2 * kKeys, kv);
             }
-            for (int it = 0; it < nitems; ++it) {
-                const int s = it & 1;
-                if (it >= 2 && !mbar_wait(&ctl.q_empty[s], ((it - 2) >> 1) & 1, wc, kSleepNs)) break;
-                const int tq = raw[list[it / G]];
-                uint8_t* st = smem + kDkvOffQ + s * 2 * kQBytes;
-                mbar_arrive_expect_tx(&ctl.q_full[s], 2 * kQBytes);
-                if (hp) {
-                    // the segment's R rows of each of the G heads
-                    const int row = ptg.base + tq * p.seg_rows;
-                    for (int hq = 0; hq < p.G; ++hq)
-                        for (int h = 0; h < 2; ++h) {
-                            const int so = h * (kRows * 128) + hq * p.seg_rows * 128;
-                            tma_load_3d(st + so, &mapQ, &ctl.q_full[s], h * 64, row, kv * p.G + hq);
-                            tma_load_3d(st + kQBytes + so, &mapDO, &ctl.q_full[s], h * 64, row, kv * p.G + hq);
-                        }
-                } else {
-                    const int row = ptg.base + tq * kRows;
-                    const int bhq = kv * G + it % G;
-                    for (int h = 0; h < 2; ++h) {
-                        tma_load_3d(st + h * (kRows * 128), &mapQ, &ctl.q_full[s], h * 64, row, bhq);
-                        tma_load_3d(st + kQBytes + h * (kRows * 128), &mapDO, &ctl.q_full[s], h * 64, row, bhq);
+            for (int x = 0; x < nh; ++x) {
+                int ri, head, h;
+                bool fst, lst;
+                half_at(x, ri, head, h, fst, lst);
+                const int s = x % kQStages;
+                if (x >= kQStages && !mbar_wait(&ctl.q_empty[s], ((x / kQStages) - 1) & 1, wc, kSleepNs)) break;
+                const int tq = raw[ri];
+                uint8_t* st = smem + kDkvOffQ + s * 2 * kQHalfBytes;
+                mbar_arrive_expect_tx(&ctl.q_full[s], 2 * kQHalfBytes);
+                // head-packed: the segment's R rows of half of the G heads
+                const int boxes = hp ? p.G / 2 : 1;
+                const int row = ptg.base + (hp ? tq * p.seg_rows : tq * kRows + h * 64);
+                for (int k = 0; k < boxes; ++k) {
+                    const int bhq = hp ? kv * p.G + h * boxes + k : kv * G + head;
+                    for (int dh2 = 0; dh2 < 2; ++dh2) {
+                        const int so = dh2 * (64 * 128) + (hp ? k * p.seg_rows * 128 : 0);
+                        tma_load_3d(st + so, &mapQ, &ctl.q_full[s], dh2 * 64, row, bhq);
+                        tma_load_3d(st + kQHalfBytes + so, &mapDO, &ctl.q_full[s], dh2 * 64, row, bhq);
                     }
                 }
             }
@@ -851,17 +918,17 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
             const uint32_t t_acc = tmem + (first ? kTmemDV : kTmemDK);
             bool ok = mbar_wait_warp(&ctl.kv_full, 0, wc, kSleepNs);
             auto issue_prod = [&](int x) -> bool {
-                const int q = x >> 1, h = x & 1, s = q & 1;
-                if (h == 0 && !mbar_wait_warp(&ctl.q_full[s], (q >> 1) & 1, wc, kSleepNs)) return false;
+                const int s = x % kQStages;
+                if (!mbar_wait_warp(&ctl.q_full[s], (x / kQStages) & 1, wc, kSleepNs)) return false;
                 tc_fence_after();
                 // B operand: Q (first issuer) or dO rows of this half, K-major
-                const uint32_t bb = smem_u32(smem + kDkvOffQ + s * 2 * kQBytes) + (first ? 0 : kQBytes);
+                const uint32_t bb = smem_u32(smem + kDkvOffQ + s * 2 * kQHalfBytes) + (first ? 0 : kQHalfBytes);
                 const uint32_t dst = t_own + (x & 1) * 128;
                 if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < kD / 16; ++k) {
                         const uint32_t oa = (k >> 2) * (2 * kKeys * 128) + (k & 3) * 32;
-                        const uint32_t ob = (k >> 2) * (kRows * 128) + h * 64 * 128 + (k & 3) * 32;
+                        const uint32_t ob = (k >> 2) * (64 * 128) + (k & 3) * 32;
                         umma_bf16(dst, smem_desc_sw128(ab + oa, 16, 1024), smem_desc_sw128(bb + ob, 16, 1024),
                                   IDESC_T, k > 0);
                     }
@@ -873,20 +940,20 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
             if (ok) ok = issue_prod(0);
             if (ok && nh > 1) ok = issue_prod(1);
             for (int x = 0; ok && x < nh; ++x) {
-                const int q = x >> 1, h = x & 1, s = q & 1, b = x & 1;
+                const int s = x % kQStages, b = x & 1;
                 if (!mbar_wait_warp(&ctl.pds_full[b], (x >> 1) & 1, wc, kSleepNs)) { ok = false; break; }
                 tc_fence_after();
                 // B operand: dO (first issuer, for dV) or Q (for dK) rows of this half, MN-major
-                const uint32_t bb = smem_u32(smem + kDkvOffQ + s * 2 * kQBytes) + (first ? kQBytes : 0);
+                const uint32_t bb = smem_u32(smem + kDkvOffQ + s * 2 * kQHalfBytes) + (first ? kQHalfBytes : 0);
                 const uint32_t a2 = t_own + b * 128;   // P^T or dS^T, in place
                 if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < 64 / 16; ++k) {
-                        const uint32_t ob = h * 64 * 128 + k * 2048;   // 16 rows = two 8-row atoms
-                        umma_bf16_ta(t_acc, a2 + k * 8, smem_desc_sw128(bb + ob, kRows * 128, 1024), IDESC_ACC,
+                        const uint32_t ob = k * 2048;   // 16 rows = two 8-row atoms
+                        umma_bf16_ta(t_acc, a2 + k * 8, smem_desc_sw128(bb + ob, 64 * 128, 1024), IDESC_ACC,
                                      (x > 0 || k > 0) ? 1u : 0u);
                     }
-                    if (h == 1) umma_commit(&ctl.q_empty[s]);
+                    umma_commit(&ctl.q_empty[s]);
                 }
                 __syncwarp();
                 // The products of half x + 2 overwrite the columns this accumulation
@@ -908,11 +975,16 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
         const int kblk = key >> 6;                // 0: block 2pr, 1: block 2pr + 1
         const uint32_t lane_addr = tmem + (static_cast<uint32_t>(warp * 32) << 16);
         bool ok = true;
+        int it = -1;   // the item
         for (int x = 0; x < nh; ++x) {
-            const int q = x >> 1, h = x & 1, si = q % kInfoStages, b = x & 1;
+            int ri, head, h;
+            bool fst, lst;
+            half_at(x, ri, head, h, fst, lst);
+            it += fst;
+            const int si = it % kInfoStages, b = x & 1;
             const float* inf = info + si * 4 * kRows;
             const uint32_t buf = lane_addr + kTmemBuf + b * 128;
-            if (h == 0 && !mbar_wait_warp(&ctl.info_full[si], (q / kInfoStages) & 1, wc, kSleepNs)) { ok = false; break; }
+            if (fst && !mbar_wait_warp(&ctl.info_full[si], (it / kInfoStages) & 1, wc, kSleepNs)) { ok = false; break; }
             if (!mbar_wait_warp(&ctl.sdp_full[b], (x >> 1) & 1, wc, kSleepNs)) { ok = false; break; }
             tc_fence_after();
             uint32_t sv[64], dv[64];
@@ -927,16 +999,15 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
             // the list, items 0 .. G-1): the rows of half h have block 2pr + h, and
             // column k is token k of it.  Head-packed: all rows of diagonal segment
             // sg are in block (sg R) / 64, column k is token (sg R) % 64 + k % R.
-            const int qi = q / G;
             bool causal;
             int toff0 = 0, rmask = 63;
             if constexpr (HP) {
-                const int sg = raw[list[qi]];
-                causal = qi < ndg && ((sg * p.seg_rows) >> 6) == 2 * pr + kblk;
+                const int sg = raw[ri];
+                causal = ri < ndg && ((sg * p.seg_rows) >> 6) == 2 * pr + kblk;
                 toff0 = (sg * p.seg_rows) & 63;
                 rmask = p.seg_rows - 1;
             } else {
-                causal = qi == 0 && h == kblk;
+                causal = ri == 0 && h == kblk;
             }
             const float2* off2 = reinterpret_cast<const float2*>(inf + kblk * kRows + h * 64);
             const float2* nd2p = reinterpret_cast<const float2*>(inf + 2 * kRows + h * 64);
@@ -975,7 +1046,7 @@ bwd_dkv_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
             tmem_wait_st();
             tc_fence_before();
             mbar_arrive_warp(&ctl.pds_full[b]);
-            if (h == 1) mbar_arrive_warp(&ctl.info_empty[si]);
+            if (lst) mbar_arrive_warp(&ctl.info_empty[si]);
         }
         if (ok && mbar_wait_warp(&ctl.fin, 0, wc, kSleepNs)) {
             tc_fence_after();
@@ -1221,10 +1292,12 @@ cudaError_t launch_attn_bwd(const AttnBwdArgs& a, const KernelEnv& env, const ch
         }
         if (e != cudaSuccess) { *err = "cudaFuncSetAttribute(bwd)"; return e; }
     }
-    CUtensorMap mq, mdo, mk, mv, mk2, mv2;
+    CUtensorMap mq, mdo, mk, mv, mk2, mv2, mqh, mdoh;
     const bool hp = a.seg_rows > 0;   // head-packed tiles: the Q / dO boxes are one head's seg_rows rows
     if (make_tmap_bf16_3d(&mq, a.Q, kD, a.N, a.BH, 64, hp ? a.seg_rows : kRows) != 0 ||
         make_tmap_bf16_3d(&mdo, a.dO, kD, a.N, a.BH, 64, hp ? a.seg_rows : kRows) != 0 ||
+        make_tmap_bf16_3d(&mqh, a.Q, kD, a.N, a.BH, 64, hp ? a.seg_rows : 64) != 0 ||   // pass 2: by halves
+        make_tmap_bf16_3d(&mdoh, a.dO, kD, a.N, a.BH, 64, hp ? a.seg_rows : 64) != 0 ||
         make_tmap_bf16_3d(&mk, a.K, kD, a.N, BHkv, 64, kKeys) != 0 ||
         make_tmap_bf16_3d(&mv, a.V, kD, a.N, BHkv, 64, kKeys) != 0 ||
         make_tmap_bf16_3d(&mk2, a.K, kD, a.N, BHkv, 64, 2 * kKeys) != 0 ||
@@ -1250,6 +1323,7 @@ cudaError_t launch_attn_bwd(const AttnBwdArgs& a, const KernelEnv& env, const ch
     p.inv_pos = a.inv_pos;
     p.slot_off = a.slot_off;
     p.offs = a.offs;
+    p.live = a.live;
     p.tiles = a.tiles;
     p.ntiles = a.ntiles;
     p.tile_off = a.tile_off;
@@ -1289,7 +1363,7 @@ cudaError_t launch_attn_bwd(const AttnBwdArgs& a, const KernelEnv& env, const ch
         // inverted lists of the KV groups' union lists
         e = cudaMemsetAsync(a.inv_cnt, 0, static_cast<size_t>(gtiles) * 4, env.stream);
         if (e != cudaSuccess) { *err = "backward list counts"; return e; }
-        const unsigned gb = static_cast<unsigned>((srcs + 255) / 256);
+        const unsigned gb = static_cast<unsigned>((srcs * 32 + 255) / 256);
         const int32_t* uidx = hp ? a.seg_union_idx : a.union_idx;
         const int32_t* ucnt = hp ? a.seg_union_cnt : a.union_cnt;
         const int ustride = hp ? a.seg_cap : a.C;
@@ -1302,10 +1376,10 @@ cudaError_t launch_attn_bwd(const AttnBwdArgs& a, const KernelEnv& env, const ch
         if (e != cudaSuccess) { *err = "backward inverted lists"; return e; }
         // pass 2: one CTA per (KV group, key pair)
         const dim3 g2(static_cast<unsigned>(gtiles));
-        if (hp && outer) bwd_dkv_kernel<true, true><<<g2, kThreadsD, kDkvSmem, env.stream>>>(mq, mdo, mk2, mv2, p);
-        else if (hp) bwd_dkv_kernel<true, false><<<g2, kThreadsD, kDkvSmem, env.stream>>>(mq, mdo, mk2, mv2, p);
-        else if (outer) bwd_dkv_kernel<false, true><<<g2, kThreadsD, kDkvSmem, env.stream>>>(mq, mdo, mk2, mv2, p);
-        else bwd_dkv_kernel<false, false><<<g2, kThreadsD, kDkvSmem, env.stream>>>(mq, mdo, mk2, mv2, p);
+        if (hp && outer) bwd_dkv_kernel<true, true><<<g2, kThreadsD, kDkvSmem, env.stream>>>(mqh, mdoh, mk2, mv2, p);
+        else if (hp) bwd_dkv_kernel<true, false><<<g2, kThreadsD, kDkvSmem, env.stream>>>(mqh, mdoh, mk2, mv2, p);
+        else if (outer) bwd_dkv_kernel<false, true><<<g2, kThreadsD, kDkvSmem, env.stream>>>(mqh, mdoh, mk2, mv2, p);
+        else bwd_dkv_kernel<false, false><<<g2, kThreadsD, kDkvSmem, env.stream>>>(mqh, mdoh, mk2, mv2, p);
         e = cudaGetLastError();
         if (e != cudaSuccess) { *err = "backward pass 2"; return e; }
     }

@@ -694,7 +694,7 @@ sas_status sas_attention_bwd(sas_handle* h, const void* Q, const void* K, const 
         const size_t per_tile = h->varlen ? 2 * static_cast<size_t>(tseq) : static_cast<size_t>(h->T + 1);
         const size_t bound = tiles * per_tile * 128 * 4;
         if (e == cudaSuccess && bound <= (static_cast<size_t>(8) << 30)) {
-            cudaError_t eb = alloc(&h->bwd_offs, bound);
+            cudaError_t eb = alloc(&h->bwd_offs, bound + bound / 128);   // + 4 `live` bytes a slot
             if (eb == cudaSuccess) {
                 h->bwd_offs_bytes = bound;
                 h->bwd_offs_bound = true;
@@ -823,11 +823,12 @@ sas_status sas_attention_bwd(sas_handle* h, const void* Q, const void* K, const 
         cudaFree(h->bwd_offs);
         h->bwd_offs = nullptr;
         h->bwd_offs_bytes = 0;
-        e = alloc(&h->bwd_offs, need);
+        e = alloc(&h->bwd_offs, need + need / 128);
         if (e != cudaSuccess) return cuda_fail(h, e, "backward offsets");
         h->bwd_offs_bytes = need;
     }
     a.offs = h->bwd_offs;
+    a.live = reinterpret_cast<uint8_t*>(h->bwd_offs) + h->bwd_offs_bytes;
     e = timed_launch(h, 6, s, [&] { return sas::launch_attn_bwd(a, env, &err); });
     if (e != cudaSuccess) return cuda_fail(h, e, err);
     // all its kernels: slot count and scan, pass 1, the inverted lists (count, scan,
