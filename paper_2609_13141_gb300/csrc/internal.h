@@ -94,7 +94,14 @@ struct SelectArgs {
     // full*: a noise table [BH][N][C] added to the scores before the gate and
     // the Top-K (null otherwise)
     const float* noise;
+    // head-packed attention tiles (as in AttnArgs; seg_rows = 0: none): segment
+    // unions with row stride seg_cap, written by the given-scores selection
+    int seg_rows, nseg, seg_cap;
+    int32_t* seg_union_idx;
+    int32_t* seg_union_cnt;
 };
+// Whether launch_select writes the segment unions itself (else launch_seg_unions).
+bool select_builds_segments(const SelectArgs& a);
 cudaError_t launch_select(const SelectArgs& a, const KernelEnv& env, const char** err);
 // Builds the tile table of packed sequences cu[0..S] (device offsets) with
 // sequences of at most max_len tokens within Ncap rows; bad offsets set the

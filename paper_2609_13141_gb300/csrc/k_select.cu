@@ -23,7 +23,8 @@
 // length, so blocks and causality restart at every sequence.
 //
 // Two score sources:
-//   * scores given: 32x32 score sub-tiles are staged through shared memory
+//   * scores given: a warp per row (select_rows_kernel); rows of more than 1280
+//     blocks one thread each, 32x32 score sub-tiles staged through shared memory
 //     with coalesced 128-byte row loads;
 //   * learned selector: on the tensor cores, one thread first projects the
 //     tile's 128 queries (q~ = Q Wq^T into TMEM; under GQA q~ = Wq_g [q_0; ...;
@@ -534,6 +535,285 @@ __global__ void __launch_bounds__(128, 3) select_given_kernel(SelParams p) {
     if (warp == 0)
         compact_union(bitmap, diag, p.union_idx + (static_cast<long long>(bh) * p.T + geo.slot) * p.C,
                       p.union_cnt + static_cast<long long>(bh) * p.T + geo.slot);
+}
+
+// Scores given, up to kRowsMaxC blocks: eight lanes per row, four rows per warp.
+// The rows come to shared memory by coalesced asynchronous copies and every pass
+// over them is a short loop, so the work does not depend on how neighbouring rows'
+// selections differ, and what a row costs whatever its length (reductions, bracket
+// updates, addresses) is shared by four.  The K-th largest score is bracketed: a
+// first guess from the mean and deviation of the row's first 128 scores (a normal
+// sample's K-th largest), one Newton step, then interpolation on the counts with a
+// midpoint every third step, and past kValueSteps counts bisection of the float
+// order, which ends at a value shared by the boundary blocks: ties then go to the
+// lower blocks.  NaN ranks as replace-the-worst has it: one among the first K blocks
+// stays, a later one never enters.
+// At 8 groups x 32768 rows, K = 32 (268 MB of scores, 40 us at the copy rate): 207 us,
+// 640 instructions a row, 70% of the issue slots; a thread per row and the segments'
+// lists in a launch of their own took 343 + 58.
+// One CTA per 128-row tile also builds the tile's union list and, for head-packed
+// attention tiles (seg_rows > 0), the lists of its segments of seg_rows tokens.
+constexpr int kRowsMaxC = 1280;   // eight warps' rows fill an SM's shared memory
+constexpr int kRowsTwoC = 704;    // two such CTAs fit
+constexpr int kRowsMinC = 64;
+constexpr int kValueSteps = 14;
+
+// order-preserving whole numbers; -0 and +0 share one
+__device__ __forceinline__ uint32_t float_order(float f) {
+    const uint32_t u = __float_as_uint(f);
+    return (u & 0x80000000u) ? 0x80000000u - (u & 0x7fffffffu) : 0x80000000u + u;
+}
+__device__ __forceinline__ float order_float(uint32_t k) {
+    return __uint_as_float(k >= 0x80000000u ? k - 0x80000000u : (0x80000000u - k) | 0x80000000u);
+}
+__device__ __forceinline__ float row_sum(float v) {   // over a row's eight lanes
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// A normal sample's K-th largest of n: its deviate z and sqrt(2 pi) exp(z^2 / 2) / n,
+// the reciprocal density of the count there.
+struct TailGuess {
+    float z, inv_density;
+};
+__device__ __forceinline__ TailGuess tail_guess(int n, int K) {
+    const float f = 1.f / static_cast<float>(n);
+    const float z = 1.41421356f * erfinvf(1.f - 2.f * static_cast<float>(K) * f);
+    return {z, 2.50662827f * fast_exp2(0.72134752f * z * z) * f};
+}
+
+__host__ __device__ __forceinline__ int rows_stride(int C) { return ((C + 31) & ~31) + 8; }   // + 8: rows on other banks
+
+__global__ void __launch_bounds__(512, 2) select_rows_kernel(SelParams p, int vec, int seg_rows, int nseg,
+                                                                   int seg_cap, int32_t* seg_idx, int32_t* seg_cnt) {
+    // per warp four rows and their K kept blocks; then [segments of the tile][C rounded up to 16] bytes
+    extern __shared__ __align__(16) uint8_t rows_smem[];
+    if (p.tiles != nullptr && static_cast<int>(blockIdx.x / p.BH) >= __ldg(p.ntiles)) return;   // spare slot
+    const TileGeo geo = tile_geo(p);
+    const int t = geo.t, bh = head_of_block(p.BH), K = p.topk;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane & 7, rr = lane >> 3;
+    const int nwarps = blockDim.x >> 5;   // 8 or 16
+    const int stride = rows_stride(p.C), Cp = (p.C + 15) & ~15;
+    float* x = reinterpret_cast<float*>(rows_smem) + warp * (4 * stride + 4 * K) + rr * stride;
+    int32_t* kept = reinterpret_cast<int32_t*>(x + (4 - rr) * stride) + rr * K;
+    uint8_t* seen = rows_smem + static_cast<size_t>(nwarps) * (4 * stride + 4 * K) * 4;
+    const int R = seg_rows > 0 ? seg_rows : kRows;   // rows per byte map
+    const int maps = kRows / R;
+    for (int w = threadIdx.x; w < maps * Cp / 4; w += blockDim.x) reinterpret_cast<uint32_t*>(seen)[w] = 0u;
+    __syncthreads();
+    const int per_warp = kRows / nwarps;
+    const int r0 = warp * per_warp, i0 = t * kRows + r0;
+    const int rows = K > 0 ? max(0, min(per_warp, geo.n - i0)) : 0;
+    const uint32_t pick = static_cast<uint32_t>(rr | ((rr + 4) << 4));   // byte rr of two ballots
+    TailGuess tg{0.f, 0.f};
+    int gC = -1;
+#pragma unroll 1
+    for (int k = 0; k < rows; k += 4) {
+        const int Ci = (i0 + k) >> 6;   // the same for the four rows
+        const bool own = k + rr < rows;
+        const long long row = static_cast<long long>(bh) * p.N + geo.base + i0 + min(k + rr, rows - 1);
+        const float* src = p.scores + row * p.C;
+        if (vec) {
+            for (int m = 4 * sub; m < Ci; m += 32) cp_async16(x + m, src + m);
+        } else {
+            for (int m = sub; m < Ci; m += 8) cp_async4(x + m, src + m);
+        }
+        cp_async_commit();
+        if (Ci != gC && Ci > K) tg = tail_guess(Ci, K);
+        gC = Ci;
+        const int groups = (Ci + 31) >> 5;
+        cp_async_wait<0>();
+        __syncwarp();
+        // padding (and what a 16-byte copy brought past the history)
+        for (int m = Ci + sub; m < 32 * groups; m += 8) x[m] = -CUDART_INF_F;
+        if (p.noise != nullptr) {
+            const float* nz = p.noise + row * p.C;
+            for (int m = sub; m < Ci; m += 8) x[m] = __fadd_rn(x[m], __ldg(nz + m));   // full*: s~ = s + eps in fp32
+        }
+        __syncwarp();
+        const float4* xv = reinterpret_cast<const float4*>(x) + sub;
+        float mx = -CUDART_INF_F;
+#pragma unroll 4
+        for (int j = 0; j < groups; ++j) {
+            const float4 v = xv[8 * j];
+            mx = fmaxf(max3f(mx, v.x, v.y), fmaxf(v.z, v.w));
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        float ex = 0.f;
+#pragma unroll 2
+        for (int j = 0; j < groups; ++j) {
+            const float4 v = xv[8 * j];
+            ex += (fast_exp2((v.x - mx) * kLog2e) + fast_exp2((v.y - mx) * kLog2e)) +
+                  (fast_exp2((v.z - mx) * kLog2e) + fast_exp2((v.w - mx) * kLog2e));
+        }
+        ex = row_sum(ex);
+        const float lse = mx + logf(ex);
+        const bool odd = __any_sync(0xffffffffu, !(ex == ex)) != 0;   // NaN (or an infinite maximum) in some row
+        if (odd) {
+            for (int m = sub; m < Ci; m += 8)
+                if (!(x[m] == x[m])) x[m] = m < K ? CUDART_INF_F : -CUDART_INF_F;
+            if (!(ex == ex)) mx = CUDART_INF_F;
+            __syncwarp();
+        }
+        // keep x >= hi (none before a bound above is found), and of the others x >= lo the first `ties`
+        float lo = -CUDART_INF_F, hi = -CUDART_INF_F;   // Ci <= K: all
+        bool above = true;
+        int ties = 0;
+        if (Ci > K) {
+            const int ns = min(Ci, 128);
+            float sum = 0.f, sq = 0.f;
+            for (int j = 0; 32 * j < ns; ++j) {
+                const float4 v = xv[8 * j];
+                const int m = 32 * j + 4 * sub;
+                const float d0 = m < ns ? v.x - mx : 0.f, d1 = m + 1 < ns ? v.y - mx : 0.f;
+                const float d2 = m + 2 < ns ? v.z - mx : 0.f, d3 = m + 3 < ns ? v.w - mx : 0.f;
+                sum += (d0 + d1) + (d2 + d3);
+                sq += fmaf(d0, d0, d1 * d1) + fmaf(d2, d2, d3 * d3);
+            }
+            const float inv_ns = 1.f / static_cast<float>(ns);
+            const float mean = row_sum(sum) * inv_ns;
+            const float sd = sqrtf(fmaxf(fmaf(-mean, mean, row_sum(sq) * inv_ns), 0.f));
+            uint32_t khi = float_order(mx) + 1u;   // no block there, Ci at lo
+            hi = mx < CUDART_INF_F ? order_float(khi) : mx;
+            above = false;
+            int clo = Ci, chi = 0;
+            float th = mx + mean + sd * tg.z;
+            bool done = false;
+#pragma unroll 1
+            for (int it = 0; it < 64; ++it) {   // at most kValueSteps + 33
+                if (!done && (it >= kValueSteps || !(th > lo && th < hi))) {
+                    const uint32_t klo = float_order(lo);
+                    if (khi - klo <= 1u) {   // only blocks of score lo between the brackets
+                        ties = K - chi;
+                        done = true;
+                    } else {
+                        th = order_float(klo + ((khi - klo) >> 1));
+                    }
+                }
+                if (__all_sync(0xffffffffu, done)) break;
+                int c = 0;
+#pragma unroll 4
+                for (int j = 0; j < groups; ++j) {
+                    const float4 w = xv[8 * j];
+                    c += (w.x >= th ? 1 : 0) + (w.y >= th ? 1 : 0) + (w.z >= th ? 1 : 0) + (w.w >= th ? 1 : 0);
+                }
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+                if (!done) {
+                    if (c > K) {
+                        lo = th;
+                        clo = c;
+                    } else {
+                        hi = th;
+                        khi = float_order(th);
+                        chi = c;
+                        above = true;
+                        done = c == K;
+                    }
+                    if (it == 0 || clo == Ci)   // Newton on a normal tail count, until something is known below
+                        th += static_cast<float>(c - K - (it > 0 ? 1 : 0)) * sd * tg.inv_density;
+                    else if (it % 3 == 2)
+                        th = 0.5f * (lo + hi);
+                    else
+                        th = lo + (hi - lo) * __fdividef(static_cast<float>(clo - K), static_cast<float>(clo - chi));
+                }
+            }
+        }
+        // kept blocks in order: the masks of eight 32-block groups, one per lane of the
+        // row, then each lane lists its own
+        const bool some_ties = __any_sync(0xffffffffu, ties > 0) != 0;
+        uint8_t* mark = seen + ((r0 + min(k + rr, rows - 1)) / R) * Cp;
+        int pos = 0;
+#pragma unroll 1
+        for (int g0 = 0; g0 < groups; g0 += 8) {
+            uint32_t mine = 0;
+            const int ng = min(8, groups - g0);
+#pragma unroll 2
+            for (int g = 0; g < ng; ++g) {
+                const float* xs = x + 32 * (g0 + g) + sub;
+                const float v0 = xs[0], v1 = xs[8], v2 = xs[16], v3 = xs[24];
+                const uint32_t b0 = __ballot_sync(0xffffffffu, v0 >= hi), b1 = __ballot_sync(0xffffffffu, v1 >= hi);
+                const uint32_t b2 = __ballot_sync(0xffffffffu, v2 >= hi), b3 = __ballot_sync(0xffffffffu, v3 >= hi);
+                uint32_t mask = __byte_perm(__byte_perm(b0, b1, pick), __byte_perm(b2, b3, pick), 0x5410);
+                if (!above) mask = 0u;
+                if (some_ties) {
+                    const uint32_t e0 = __ballot_sync(0xffffffffu, v0 >= lo), e1 = __ballot_sync(0xffffffffu, v1 >= lo);
+                    const uint32_t e2 = __ballot_sync(0xffffffffu, v2 >= lo), e3 = __ballot_sync(0xffffffffu, v3 >= lo);
+                    uint32_t eq = __byte_perm(__byte_perm(e0, e1, pick), __byte_perm(e2, e3, pick), 0x5410) & ~mask;
+                    for (; eq != 0u && ties > 0; --ties) {
+                        mask |= eq & (0u - eq);
+                        eq &= eq - 1u;
+                    }
+                }
+                if (g == sub) mine = mask;
+            }
+            const int lim = Ci - 32 * (g0 + sub);   // the padding is not a block
+            if (lim < 32) mine &= lim > 0 ? (1u << lim) - 1u : 0u;
+            const int cnt = __popc(mine);
+            int incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+                const int up = __shfl_up_sync(0xffffffffu, incl, o, 8);
+                if (sub >= o) incl += up;
+            }
+            int e = pos + incl - cnt;
+            pos += __shfl_sync(0xffffffffu, incl, 7, 8);
+            for (; mine != 0u && e < K; ++e) {
+                const int m = 32 * (g0 + sub) + __ffs(mine) - 1;
+                mine &= mine - 1u;
+                kept[e] = m;
+                mark[m] = 1;
+            }
+        }
+        __syncwarp();
+        if (own) {
+            int32_t* si = p.sel_idx + row * K;
+            float* sl = p.sel_logg + row * K;
+            for (int e = sub; e < K; e += 8) {
+                const bool in = e < pos;   // short histories
+                const int m = in ? kept[e] : -1;
+                float g = 0.f;
+                if (in) {
+                    float s = x[m];
+                    if (odd) s = p.noise != nullptr ? __fadd_rn(__ldg(src + m), __ldg(p.noise + row * p.C + m)) : __ldg(src + m);
+                    g = staged_gate(s, lse, p.gate_act);
+                    if (p.gate_act == 1) g = log_sigmoid(g);
+                }
+                si[e] = m;
+                sl[e] = g;
+            }
+        }
+        __syncwarp();   // before the next rows overwrite these
+    }
+    __syncthreads();
+    // union lists: warp w the segments w, w + warps, ...; the last also the tile's own
+    if (seg_rows > 0)
+        for (int g = warp; g < maps; g += nwarps) {
+            const int sg = p.tiles == nullptr ? t * maps + g : geo.slot * maps + g;
+            if (sg >= nseg) break;
+            const long long item = static_cast<long long>(bh) * nseg + sg;
+            // a segment's kept blocks lie below its own block
+            compact_union_bytes(seen + g * Cp, min((t * kRows + g * R) >> 6, p.C), seg_idx + item * seg_cap,
+                                seg_cnt + item);
+        }
+    if (warp == nwarps - 1) {
+        const long long tb = static_cast<long long>(bh) * p.T + geo.slot;
+        const int diag = min(2 * t, p.C);
+        int32_t* out = p.union_idx + tb * p.C;
+        int base = 0;
+        for (int m0 = 0; m0 < diag; m0 += 32) {
+            const int m = m0 + lane;
+            bool set = false;
+            if (m < diag)
+                for (int g = 0; g < maps; ++g) set = set || seen[g * Cp + m] != 0;
+            const uint32_t bal = __ballot_sync(0xffffffffu, set);
+            if (set) out[base + __popc(bal & ((1u << lane) - 1u))] = m;
+            base += __popc(bal);
+        }
+        if (lane == 0) p.union_cnt[tb] = base;
+    }
 }
 
 // --------------------------------------------------------- learned selector
@@ -1322,6 +1602,30 @@ cudaError_t launch_proj(const SelectArgs& a, const SelParams& p, const KernelEnv
     return cudaErrorInvalidValue;
 }
 
+// A warp takes its rows one batch of four after another, about 3 us each alone, so
+// sixteen warps where their rows fit several times over (4096 x 8 heads, K = 32: 45.7 us
+// with four warps, 19.9 with sixteen) or where a tile has the SM to itself; else eight
+// (32768 x 8, K = 32: 219 us with four, 207 with eight: 24 warps on an SM for 20).
+int rows_warps(const SelectArgs& a) {
+    return a.C <= 128 || (a.C <= 512 && a.BH * a.T <= device_sm_count()) ? 16 : 8;
+}
+
+cudaError_t launch_rows(const SelectArgs& a, const SelParams& p, const KernelEnv& env, const char** err) {
+    const int maps = a.seg_rows > 0 ? kRows / a.seg_rows : 1;
+    const int nwarps = rows_warps(a);
+    const size_t smem = static_cast<size_t>(nwarps) * (4 * rows_stride(a.C) + 4 * a.topk) * 4 +
+                        static_cast<size_t>(maps) * ((a.C + 15) & ~15);
+    cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(select_rows_kernel), smem);
+    if (e != cudaSuccess) { *err = "cudaFuncSetAttribute(select_rows)"; return e; }
+    // 16-byte copies need aligned rows and whole groups of four within them
+    const int vec = a.C % 4 == 0 && (reinterpret_cast<uintptr_t>(a.scores) & 15u) == 0 ? 1 : 0;
+    select_rows_kernel<<<dim3(a.BH * a.T), 32 * nwarps, smem, env.stream>>>(
+        p, vec, a.seg_rows, a.nseg, a.seg_cap, a.seg_union_idx, a.seg_union_cnt);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) *err = "select launch";
+    return e;
+}
+
 template <bool REG, bool NOISE>
 cudaError_t launch_given(const SelectArgs& a, const SelParams& p, const KernelEnv& env, const char** err) {
     const size_t smem = smem_topk_bytes(a.topk) + staging_bytes(a.topk) + bitmap_bytes(a.C);
@@ -1503,6 +1807,20 @@ cudaError_t launch_row_lse(const float* scores, int N, int C, long long rows, fl
     return cudaGetLastError();
 }
 
+// Which kernel selects from given scores (us, thread per row -> eight lanes per row;
+// d = 64, normal scores).  K <= 32: a thread's list is in registers, and up to 2048
+// tokens there is little to replace and its shorter chain wins (2048 x 32 heads, K = 4:
+// 22.9 against 26.7; K = 32: 15.7 / 16.6), from 4096 on the rows kernel (4096 x 8,
+// K = 16: 22.0 / 18.3; 8192 x 2, K = 32: 34.0 / 18.5; 16384 x 4, K = 32: 89.4 / 44.3;
+// 40960 x 2, K = 4: 137 / 97), until its rows leave room for one CTA of eight warps on
+// an SM (81920 x 2, K = 16: 414 / 444).  K > 32: the thread's list is in shared memory
+// and the rows kernel is faster at every length it holds (4096 x 8, K = 64: 23.3 / 15.0;
+// 8192 x 16: 389 / 59; 81920 x 2: 3453 / 475).
+bool select_builds_segments(const SelectArgs& a) {
+    if (a.scores == nullptr || a.score_scale != 1.f || a.full_lse != nullptr) return false;
+    return a.topk > 32 ? a.C <= kRowsMaxC : a.C >= kRowsMinC && a.C <= kRowsTwoC;
+}
+
 cudaError_t launch_select(const SelectArgs& a, const KernelEnv& env, const char** err) {
     SelParams p;
     p.BH = a.BH; p.N = a.N; p.C = a.C; p.T = a.T; p.F = a.F; p.topk = a.topk;
@@ -1526,6 +1844,7 @@ cudaError_t launch_select(const SelectArgs& a, const KernelEnv& env, const char*
     }
 
     const bool reg = a.topk <= 32;
+    if (a.scores != nullptr && select_builds_segments(a)) return launch_rows(a, p, env, err);
     if (a.scores != nullptr) {
         if (a.noise != nullptr)
             return reg ? launch_given<true, true>(a, p, env, err) : launch_given<false, true>(a, p, env, err);

@@ -452,13 +452,15 @@ sas_status attention_fwd(sas_handle* h, const void* Q, const void* K, const void
     sa.sel_idx = out_idx; sa.sel_logg = out_lg;
     sa.union_idx = h->union_idx; sa.union_cnt = h->union_cnt;
     sa.noise = noise;
+    sa.seg_rows = h->seg_rows; sa.nseg = h->nseg; sa.seg_cap = h->seg_cap;
+    sa.seg_union_idx = h->seg_union_idx; sa.seg_union_cnt = h->seg_union_cnt;
     if (h->full) {
         sa.full_lse = h->full_lse;
         sa.full_table = h->full_table;
     }
     e = timed_launch(h, 2, s, [&] { return sas::launch_select(sa, env, &err); });
     if (e != cudaSuccess) return cuda_fail(h, e, err);
-    if (h->seg_rows > 0) {
+    if (h->seg_rows > 0 && !sas::select_builds_segments(sa)) {
         // the segment unions of the head-packed attention tiles (timed with the selection)
         e = timed_launch(h, 2, s, [&] {
             return sas::launch_seg_unions(out_idx, h->BHkv, c.N, h->C, c.topk, h->seg_rows, h->nseg, h->seg_union_idx,
@@ -564,9 +566,11 @@ sas_status sas_attention_fwd_varlen(sas_handle* h, const int32_t* cu_seqlens, in
     sa.sel_idx = out_idx; sa.sel_logg = out_lg;
     sa.union_idx = h->union_idx; sa.union_cnt = h->union_cnt;
     sa.tiles = h->tiles; sa.ntiles = h->ntiles;
+    sa.seg_rows = h->seg_rows; sa.nseg = h->nseg; sa.seg_cap = h->seg_cap;
+    sa.seg_union_idx = h->seg_union_idx; sa.seg_union_cnt = h->seg_union_cnt;
     e = timed_launch(h, 2, s, [&] { return sas::launch_select(sa, env, &err); });
     if (e != cudaSuccess) return cuda_fail(h, e, err);
-    if (h->seg_rows > 0) {
+    if (h->seg_rows > 0 && !sas::select_builds_segments(sa)) {
         // the segment unions of the head-packed attention tiles (timed with the selection)
         e = timed_launch(h, 2, s, [&] {
             return sas::launch_seg_unions(out_idx, h->BHkv, c.N, h->C, c.topk, h->seg_rows, h->nseg, h->seg_union_idx,
