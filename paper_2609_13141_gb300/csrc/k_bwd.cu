@@ -1123,15 +1123,20 @@ __global__ void __launch_bounds__(256) bwd_dense_unions_kernel(int32_t* uidx, in
 // independent gates: ds_m = dlogg_m d(log g_m)/ds_m on kept blocks only
 // (act 1, sigmoid: dlogg_m (1 - g_m) = -dlogg_m expm1(log g_m); act 2, raw
 // logit: dlogg_m).  One warp per row, every load of the row
-// issued first (the row's scores are held in registers when C <= 32 NCH):
+// issued first (the row's scores are held in registers when C <= 128 NV):
 // the log-normaliser comes back from the first kept entry (log g_m = s_m -
 // LSE of the scores, Eq. normalized_log_gate), the kept dlogg values are
 // scattered into the warp's C floats of shared memory.
-template <int NCH>
+// A stream over the score matrices: rows move as 16-byte words where they are aligned
+// (VEC: C a multiple of 4, both matrices on 16 bytes), else word by word.  24 heads x
+// 16896 rows of 264 blocks, 0.64 GB (112 us with the lists at the copy rate): 172 us,
+// 228 word by word; what is left is the wait for each row's loads (fewer registers
+// for more warps spill: 185 us at six CTAs per SM, 197 at eight).
+template <int NV, bool VEC>
 __global__ void __launch_bounds__(256)
 bwd_ds_kernel(const float* scores, const int32_t* sel_idx, const float* sel_logg, const float* dlogg, float* ds,
               int N, int C, int topk, int train, int act, int chunks, const int4* tiles, const int* ntiles) {
-    extern __shared__ float dsh[];   // per warp: C floats (the row's kept dlogg, scattered)
+    extern __shared__ __align__(16) float dsh[];   // per warp: C floats (the row's kept dlogg, scattered)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // CTA = (head, run of blockDim / 32 rows of it): one division per CTA.
     // Packed sequences: chunks = tile slots x runs per 128-row tile, and i is
@@ -1159,12 +1164,21 @@ bwd_ds_kernel(const float* scores, const int32_t* sel_idx, const float* sel_logg
     const int nsel = train ? min(topk, c) : 0;
     const float* s = scores + w * C;
     float* out = ds + w * C;
-    float sv[NCH > 0 ? NCH : 1];
-    if (NCH > 0) {
+    float4 sv[NV > 0 ? NV : 1];   // VEC: blocks 128 q + 4 lane ..; else 128 q + lane, + 32, + 64, + 96
+    if (NV > 0) {
 #pragma unroll
-        for (int q = 0; q < NCH; ++q) {
-            const int m = lane + 32 * q;
-            sv[q] = m < c ? __ldg(s + m) : 0.f;
+        for (int q = 0; q < NV; ++q) {
+            sv[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (VEC) {
+                const int m = 128 * q + 4 * lane;
+                if (m < c) sv[q] = __ldg(reinterpret_cast<const float4*>(s + m));
+            } else {
+                const int m = 128 * q + lane;
+                if (m < c) sv[q].x = __ldg(s + m);
+                if (m + 32 < c) sv[q].y = __ldg(s + m + 32);
+                if (m + 64 < c) sv[q].z = __ldg(s + m + 64);
+                if (m + 96 < c) sv[q].w = __ldg(s + m + 96);
+            }
         }
     }
     const int32_t* ix = sel_idx + w * topk;
@@ -1175,7 +1189,11 @@ bwd_ds_kernel(const float* scores, const int32_t* sel_idx, const float* sel_logg
     const float v0 = lane < nsel ? __ldg(dl + lane) * dlds(lane) : 0.f;
     const int i0 = lane < nsel ? __ldg(ix + lane) : 0;
     const float lg0 = nsel > 0 ? __ldg(lgr) : 0.f;
-    for (int m = lane; m < C; m += 32) add[m] = 0.f;
+    if constexpr (VEC) {
+        for (int m = 4 * lane; m < c; m += 128) *reinterpret_cast<float4*>(add + m) = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+        for (int m = lane; m < c; m += 32) add[m] = 0.f;
+    }
     __syncwarp();
     float sum = v0;
     if (lane < nsel) add[i0] = v0;   // kept blocks are distinct
@@ -1186,42 +1204,44 @@ bwd_ds_kernel(const float* scores, const int32_t* sel_idx, const float* sel_logg
     }
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (act != 0) sum = 0.f;   // independent gates: no coupling term
-    // LSE = s_m0 - log g_m0 for the first kept block m0 (< c, so in registers)
+    // LSE = s_m0 - log g_m0 for the first kept block m0 (its line is in L1)
     const int m0 = __shfl_sync(0xffffffffu, i0, 0);
-    float s0;
-    if (NCH > 0) {
-        float mine = 0.f;
-#pragma unroll
-        for (int q = 0; q < NCH; ++q)
-            if (q == (m0 >> 5)) mine = sv[q];
-        s0 = __shfl_sync(0xffffffffu, mine, m0 & 31);
-    } else {
-        s0 = nsel > 0 ? __ldg(s + m0) : 0.f;
-    }
-    const float lse = s0 - lg0;
+    const float lse = (nsel > 0 && static_cast<unsigned>(m0) < static_cast<unsigned>(c) ? __ldg(s + m0) : 0.f) - lg0;
     __syncwarp();
-    if (NCH > 0) {
-#pragma unroll
-        for (int q = 0; q < NCH; ++q) {
-            const int m = lane + 32 * q;
-            if (m < C) {
-                float v = 0.f;
-                if (m < c) {
-                    v = add[m];
-                    if (sum != 0.f) v -= __expf(sv[q] - lse) * sum;
-                }
-                out[m] = v;
+    auto grad = [&](int m, float x, float kept) {
+        if (m >= c) return 0.f;
+        return sum != 0.f ? kept - __expf(x - lse) * sum : kept;
+    };
+    if constexpr (VEC) {
+        auto put = [&](int m, const float4& x) {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (m < c) {
+                const float4 a = *reinterpret_cast<const float4*>(add + m);
+                v = make_float4(grad(m, x.x, a.x), grad(m + 1, x.y, a.y), grad(m + 2, x.z, a.z), grad(m + 3, x.w, a.w));
             }
+            *reinterpret_cast<float4*>(out + m) = v;
+        };
+        if (NV > 0) {
+#pragma unroll
+            for (int q = 0; q < NV; ++q) {
+                const int m = 128 * q + 4 * lane;
+                if (m < C) put(m, sv[q]);
+            }
+        } else {
+            for (int m = 4 * lane; m < C; m += 128)
+                put(m, m < c ? __ldg(reinterpret_cast<const float4*>(s + m)) : make_float4(0.f, 0.f, 0.f, 0.f));
+        }
+    } else if (NV > 0) {
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            const int m = 128 * q + lane;
+            if (m < C) out[m] = m < c ? grad(m, sv[q].x, add[m]) : 0.f;
+            if (m + 32 < C) out[m + 32] = m + 32 < c ? grad(m + 32, sv[q].y, add[m + 32]) : 0.f;
+            if (m + 64 < C) out[m + 64] = m + 64 < c ? grad(m + 64, sv[q].z, add[m + 64]) : 0.f;
+            if (m + 96 < C) out[m + 96] = m + 96 < c ? grad(m + 96, sv[q].w, add[m + 96]) : 0.f;
         }
     } else {
-        for (int m = lane; m < C; m += 32) {
-            float v = 0.f;
-            if (m < c) {
-                v = add[m];
-                if (sum != 0.f) v -= __expf(__ldg(s + m) - lse) * sum;
-            }
-            out[m] = v;
-        }
+        for (int m = lane; m < C; m += 32) out[m] = m < c ? grad(m, __ldg(s + m), add[m]) : 0.f;
     }
 }
 
@@ -1402,15 +1422,13 @@ cudaError_t launch_attn_bwd(const AttnBwdArgs& a, const KernelEnv& env, const ch
         const int chunks = a.tiles != nullptr ? a.T * (kRows / wpc) : (a.N + wpc - 1) / wpc;
         const unsigned grid = static_cast<unsigned>(static_cast<long long>(BHkv) * chunks);
         const int train = a.mode == 0 ? 1 : 0;
-        if (a.C <= 128)
-            bwd_ds_kernel<4><<<grid, 32 * wpc, sh, env.stream>>>(a.scores, a.sel_idx, a.sel_logg, a.dlogg, a.ds, a.N,
-                                                                 a.C, a.topk, train, a.act, chunks, a.tiles, a.ntiles);
-        else if (a.C <= 384)
-            bwd_ds_kernel<12><<<grid, 32 * wpc, sh, env.stream>>>(a.scores, a.sel_idx, a.sel_logg, a.dlogg, a.ds, a.N,
-                                                                  a.C, a.topk, train, a.act, chunks, a.tiles, a.ntiles);
-        else
-            bwd_ds_kernel<0><<<grid, 32 * wpc, sh, env.stream>>>(a.scores, a.sel_idx, a.sel_logg, a.dlogg, a.ds, a.N,
-                                                                 a.C, a.topk, train, a.act, chunks, a.tiles, a.ntiles);
+        const bool vec = a.C % 4 == 0 &&
+                         ((reinterpret_cast<uintptr_t>(a.scores) | reinterpret_cast<uintptr_t>(a.ds)) & 15u) == 0;
+        auto* const kernel = a.C <= 128   ? (vec ? bwd_ds_kernel<1, true> : bwd_ds_kernel<1, false>)
+                             : a.C <= 384 ? (vec ? bwd_ds_kernel<3, true> : bwd_ds_kernel<3, false>)
+                                          : (vec ? bwd_ds_kernel<0, true> : bwd_ds_kernel<0, false>);
+        kernel<<<grid, 32 * wpc, sh, env.stream>>>(a.scores, a.sel_idx, a.sel_logg, a.dlogg, a.ds, a.N, a.C, a.topk,
+                                                   train, a.act, chunks, a.tiles, a.ntiles);
         e = cudaGetLastError();
         if (e != cudaSuccess) { *err = "backward score gradient"; return e; }
     } else if (a.ds != nullptr) {
