@@ -1747,18 +1747,21 @@ namespace {
 // tokens share one current block c (R <= 64, segments aligned), and kept
 // blocks are < c.  cap: row stride of the output lists (>= min(C, R topk)).
 // Packed sequences: segment sg is part sg % G of tile slot sg / G (G = 128 / R).
+// The segment's lists are one run of R topk words, read by all lanes at once (a lane
+// per token, one entry after another, took 37 us for 8 groups x 19000 packed tokens, K = 32;
+// now 8.4: 5 us of it the lists at the copy rate).
+// BYTES: the set is a byte per block, written without atomics (lists of neighbouring
+// tokens mostly agree); longer histories, past kSegByteC blocks, take a bit per block.
+constexpr int kSegByteC = 5120;   // eight warps' maps in 40 KB
+template <bool BYTES>
 __global__ void __launch_bounds__(256) seg_union_kernel(const int32_t* sel_idx, int BHkv, int N, int C, int topk,
                                                         int R, int nseg, int cap, int32_t* out_idx,
                                                         int32_t* out_cnt, const int4* tiles, const int* ntiles) {
-    extern __shared__ uint32_t segbits[];   // per warp: ceil(C / 32) words
+    extern __shared__ __align__(16) uint32_t segset[];   // per warp: a byte (rounded up to 16) or a bit per block
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long item = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + warp;
     if (item >= static_cast<long long>(BHkv) * nseg) return;   // no block-wide synchronisation below
     const int kv = static_cast<int>(item / nseg), sg = static_cast<int>(item - static_cast<long long>(kv) * nseg);
-    const int nw = (C + 31) >> 5;
-    uint32_t* bits = segbits + warp * nw;
-    for (int w = lane; w < nw; w += 32) bits[w] = 0u;
-    __syncwarp();
     // the segment's first token within its sequence, the sequence's first row and length
     int i0 = sg * R, base = 0, n = N;
     if (tiles != nullptr) {
@@ -1769,19 +1772,23 @@ __global__ void __launch_bounds__(256) seg_union_kernel(const int32_t* sel_idx, 
         base = v.x;
         n = v.z;
     }
-    for (int rr = lane; rr < R; rr += 32) {
-        const int i = i0 + rr;
-        if (i >= n) break;
-        const int c = i >> 6;
-        const int ne = min(topk, c);
-        const int32_t* idx = sel_idx + (static_cast<long long>(kv) * N + base + i) * topk;
-        for (int e = 0; e < ne; ++e) {
-            const int m = __ldg(idx + e);
-            if (static_cast<unsigned>(m) < static_cast<unsigned>(c)) atomicOr(&bits[m >> 5], 1u << (m & 31));
-        }
+    const int c = i0 >> 6;
+    const int nw = BYTES ? ((C + 15) & ~15) >> 2 : (C + 31) >> 5;
+    uint32_t* set = segset + warp * nw;
+    for (int w = lane; w < nw; w += 32) set[w] = 0u;
+    __syncwarp();
+    const int total = max(0, min(R, n - i0)) * topk;
+    const int32_t* idx = sel_idx + (static_cast<long long>(kv) * N + base + i0) * topk;
+#pragma unroll 4
+    for (int e = lane; e < total; e += 32) {
+        const int m = __ldg(idx + e);
+        if (static_cast<unsigned>(m) >= static_cast<unsigned>(c)) continue;   // the rest of a short list is -1
+        if constexpr (BYTES) reinterpret_cast<uint8_t*>(set)[m] = 1;
+        else atomicOr(&set[m >> 5], 1u << (m & 31));
     }
     __syncwarp();
-    compact_union(bits, i0 >> 6, out_idx + item * cap, out_cnt + item);
+    if constexpr (BYTES) compact_union_bytes(reinterpret_cast<uint8_t*>(set), min(c, C), out_idx + item * cap, out_cnt + item);
+    else compact_union(set, min(c, C), out_idx + item * cap, out_cnt + item);
 }
 
 }  // namespace
@@ -1790,13 +1797,15 @@ cudaError_t launch_seg_unions(const int32_t* sel_idx, int BHkv, int N, int C, in
                               int32_t* seg_union_idx, int32_t* seg_union_cnt, const KernelEnv& env, const int4* tiles,
                               const int* ntiles) {
     const long long items = static_cast<long long>(BHkv) * nseg;
-    const size_t smem = static_cast<size_t>(8) * ((C + 31) / 32) * 4;
+    const bool bytes = C <= kSegByteC;
+    const size_t smem = static_cast<size_t>(8) * (bytes ? (C + 15) & ~15 : (C + 31) / 32 * 4);
+    auto* const kernel = bytes ? seg_union_kernel<true> : seg_union_kernel<false>;
     if (smem > 48 * 1024) {
-        cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(seg_union_kernel), smem);
+        cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(kernel), smem);
         if (e != cudaSuccess) return e;
     }
     const int cap = min(C, seg_rows * max(topk, 1));
-    seg_union_kernel<<<static_cast<unsigned>((items + 7) / 8), 256, smem, env.stream>>>(
+    kernel<<<static_cast<unsigned>((items + 7) / 8), 256, smem, env.stream>>>(
         sel_idx, BHkv, N, C, topk, seg_rows, nseg, cap, seg_union_idx, seg_union_cnt, tiles, ntiles);
     return cudaGetLastError();
 }

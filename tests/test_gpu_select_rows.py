@@ -7,7 +7,7 @@ first) on every checked row, log-gates s - logsumexp(s) within the fp32 bound.""
 import pytest
 import torch
 
-from paper_2609_13141_gb300 import sas
+from paper_2609_13141_gb300 import sas, synth
 from tests import parity as P
 
 pytestmark = pytest.mark.gpu
@@ -144,3 +144,22 @@ def test_special_values(kind, act):
         fin = lg.isfinite()
         got = sl[0, 0, i, :k].double()
         assert float((got - lg)[fin].abs().max() if fin.any() else 0.0) <= P.LOGG_MAX_ABS, f"row {i}"
+
+
+@pytest.mark.parametrize("N", [64 * 5120, 64 * 5120 + 1])
+def test_segment_lists_of_long_histories(N):
+    """Learned selection, head-packed tiles: the segment lists' sets hold a byte per
+    block up to 5120 blocks, a bit beyond.  Each list is its tokens' distinct blocks."""
+    H, Hkv, K, d = 2, 1, 2, 64
+    g = torch.Generator(device=DEV).manual_seed(N)
+    Q, Kk, V = (torch.randn(1, h, N, d, generator=g, device=DEV).bfloat16() for h in (H, Hkv, Hkv))
+    Wq, Wk = (w.to(DEV) for w in synth.decode_selector_weights(Hkv, H // Hkv, d, d, seed=1, exact=True))
+    layer = sas.SasLayer(1, H, N, d, K, Hkv=Hkv, selector=sas.SAS_SEL_MEANPOOL_PROJ, d_sel=d)
+    _, _, si, _ = layer.attention(Q, Kk, V, Wq=Wq, Wk=Wk)
+    torch.cuda.synchronize()
+    _, blocks = sas.sas_get_attention_work(layer.h)
+    layer.close()
+    seg = torch.arange(N, device=DEV)[:, None].expand(N, K) // 64   # 64 tokens of two heads fill a tile
+    kept = si[0, 0].long()
+    pairs = torch.unique((seg * (1 << 20) + kept)[kept >= 0])
+    assert blocks == int(pairs.numel()) + -(-N // 64)
