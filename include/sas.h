@@ -300,6 +300,20 @@ sas_status sas_attention_fwd_varlen(sas_handle* h, const int32_t* cu_seqlens, in
                                     const void* Wq, const void* Wk,
                                     void* O, float* LSE, int32_t* sel_idx, float* sel_logg, void* stream);
 
+/* Fills the rows past cu[num_seqs] of tensors of the last
+ * sas_attention_fwd_varlen on the handle (of every row, if its offsets were bad),
+ * in one launch: tensor k is [heads][N][row_bytes] (row_bytes a multiple of 4, ptr
+ * 4-byte aligned), each 32-bit word of its spare rows becomes `fill`.  1 to
+ * SAS_MAX_TAILS tensors.  Graph-capturable. */
+#define SAS_MAX_TAILS 8
+typedef struct {
+    void* ptr;
+    int32_t heads;
+    int32_t row_bytes;
+    uint32_t fill;
+} sas_tail;
+sas_status sas_fill_varlen_tails(sas_handle* h, const sas_tail* tails, int32_t count, void* stream);
+
 /* Dense MLP sublayer Y = GELU(X W1^T + b1) W2^T + b2 with the exact (erf)
  * GELU.  SAS itself does not define or change the MLP; this is the plain
  * transformer MLP that completes a layer.

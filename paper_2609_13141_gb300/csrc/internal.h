@@ -105,12 +105,22 @@ bool select_builds_segments(const SelectArgs& a);
 cudaError_t launch_select(const SelectArgs& a, const KernelEnv& env, const char** err);
 // Builds the tile table of packed sequences cu[0..S] (device offsets) with
 // sequences of at most max_len tokens within Ncap rows; bad offsets set the
-// status word to SAS_ERR_INVALID_ARG and leave *ntiles = 0.  Slots are
+// status word to SAS_ERR_INVALID_ARG and leave ntiles[0] = 0.  ntiles[1] is the
+// number of rows the sequences cover (cu[S]; 0 if bad).  Slots are
 // ordered by local tile index, longest sequences first: local tile t of the
 // sequence of rank r sits at slot tile_off[t] + r (tile_off: ceil(max_len /
 // 128) + 1 ints).
 cudaError_t launch_varlen_tiles(const int32_t* cu, int S, int Ncap, int max_len, int4* tiles, int* ntiles,
                                 int* tile_off, const KernelEnv& env);
+// Spare rows ([ntiles[1], N) of every head) of `count` <= kMaxTails tensors.
+constexpr int kMaxTails = 8;
+struct TailFill {
+    uint32_t* ptr[kMaxTails];
+    int heads[kMaxTails], row_words[kMaxTails];
+    uint32_t fill[kMaxTails];
+    int count;
+};
+cudaError_t launch_varlen_tails(const TailFill& f, int N, const int* ntiles, const KernelEnv& env);
 
 // ---- a5: fused gated block-sparse attention forward.
 struct AttnArgs {

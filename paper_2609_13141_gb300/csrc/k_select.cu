@@ -23,8 +23,8 @@
 // length, so blocks and causality restart at every sequence.
 //
 // Two score sources:
-//   * scores given: a warp per row (select_rows_kernel); rows of more than 1280
-//     blocks one thread each, 32x32 score sub-tiles staged through shared memory
+//   * scores given: eight lanes per row (select_rows_kernel); short and very long
+//     rows one thread each, 32x32 score sub-tiles staged through shared memory
 //     with coalesced 128-byte row loads;
 //   * learned selector: on the tensor cores, one thread first projects the
 //     tile's 128 queries (q~ = Q Wq^T into TMEM; under GQA q~ = Wq_g [q_0; ...;
@@ -1694,7 +1694,8 @@ __global__ void __launch_bounds__(1024) varlen_tiles_kernel(const int32_t* cu, i
     __syncthreads();
     if (bad) {
         if (tid == 0) {
-            *ntiles = 0;
+            ntiles[0] = 0;
+            ntiles[1] = 0;
             atomicExch(status, kStatusBadInput);
         }
         return;
@@ -1708,7 +1709,8 @@ __global__ void __launch_bounds__(1024) varlen_tiles_kernel(const int32_t* cu, i
             off[t] = o;
             o += g;
         }
-        *ntiles = o;
+        ntiles[0] = o;
+        ntiles[1] = __ldg(cu + S);
     }
     __syncthreads();
     // first slot of every local tile index: sequence s of rank r keeps its
@@ -1737,6 +1739,41 @@ cudaError_t launch_varlen_tiles(const int32_t* cu, int S, int Ncap, int max_len,
     }
     varlen_tiles_kernel<<<1, 1024, smem, env.stream>>>(cu, S, Ncap, max_len, tmax, tiles, ntiles, tile_off,
                                                        env.status);
+    return cudaGetLastError();
+}
+
+namespace {
+
+// CTA (x, y) fills part x of head y's spare rows in each tensor.  Mostly there are
+// few: clearing whole outputs ahead of the kernels that write nearly all of them
+// again took 49 us of the 710 of a 32-head call over 19000 packed tokens (155 MB of
+// O alone), this 2 us.
+__global__ void __launch_bounds__(256) varlen_tails_kernel(TailFill f, int N, const int* ntiles) {
+    const int first = min(max(__ldg(ntiles + 1), 0), N);
+    const int head = blockIdx.y;
+    if (first >= N) return;
+    for (int k = 0; k < f.count; ++k) {
+        if (head >= f.heads[k]) continue;
+        const long long w = f.row_words[k];
+        uint32_t* p = f.ptr[k] + (static_cast<long long>(head) * N + first) * w;
+        const long long n = (N - first) * w;
+        const uint32_t v = f.fill[k];
+        const long long start = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+        const long long step = static_cast<long long>(gridDim.x) * blockDim.x;
+        if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0 && n % 4 == 0) {
+            for (long long i = start; i < n / 4; i += step) reinterpret_cast<uint4*>(p)[i] = make_uint4(v, v, v, v);
+        } else {
+            for (long long i = start; i < n; i += step) p[i] = v;
+        }
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_varlen_tails(const TailFill& f, int N, const int* ntiles, const KernelEnv& env) {
+    int heads = 1;
+    for (int k = 0; k < f.count; ++k) heads = max(heads, f.heads[k]);
+    varlen_tails_kernel<<<dim3(8, heads), 256, 0, env.stream>>>(f, N, ntiles);
     return cudaGetLastError();
 }
 

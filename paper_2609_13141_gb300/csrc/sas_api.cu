@@ -601,6 +601,30 @@ sas_status sas_attention_fwd_varlen(sas_handle* h, const int32_t* cu_seqlens, in
     return SAS_OK;
 }
 
+sas_status sas_fill_varlen_tails(sas_handle* h, const sas_tail* tails, int32_t count, void* stream) {
+    if (h == nullptr) return SAS_ERR_INVALID_ARG;
+    if (!h->varlen) return fail(h, SAS_ERR_INVALID_ARG, "handle not created for packed sequences (max_seqs = 0)");
+    static_assert(SAS_MAX_TAILS == sas::kMaxTails, "tail limits");
+    if (tails == nullptr || count < 1 || count > SAS_MAX_TAILS)
+        return fail(h, SAS_ERR_INVALID_ARG, "1 .. SAS_MAX_TAILS tensors");
+    sas::TailFill f{};
+    for (int32_t k = 0; k < count; ++k) {
+        const sas_tail& t = tails[k];
+        if (!t.ptr || !aligned4(t.ptr) || t.row_bytes < 4 || t.row_bytes % 4 != 0 || t.heads < 1 || t.heads > 65535)
+            return fail(h, SAS_ERR_INVALID_ARG, "tails: 4-byte aligned rows of whole words, 1 .. 65535 heads");
+        f.ptr[k] = static_cast<uint32_t*>(t.ptr);
+        f.heads[k] = t.heads;
+        f.row_words[k] = t.row_bytes / 4;
+        f.fill[k] = t.fill;
+    }
+    f.count = count;
+    const sas::KernelEnv env{static_cast<cudaStream_t>(stream), h->status, h->limit};
+    const cudaError_t e = sas::launch_varlen_tails(f, h->cfg.N, h->ntiles, env);
+    if (e != cudaSuccess) return cuda_fail(h, e, "spare rows");
+    h->launches += 1;
+    return SAS_OK;
+}
+
 sas_status sas_mlp_fwd(sas_handle* h, const void* X, const void* W1, const void* b1, const void* W2, const void* b2,
                        void* Y, int64_t T, int64_t D, int64_t F, void* stream) {
     if (h == nullptr) return SAS_ERR_INVALID_ARG;

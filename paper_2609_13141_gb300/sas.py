@@ -61,6 +61,11 @@ SAS_DECODE_NUM_KERNEL_KINDS = 4
 DECODE_KERNEL_KINDS = ["prep", "select", "attention", "summarize"]
 
 
+class SasTail(ctypes.Structure):
+    _fields_ = [("ptr", ctypes.c_void_p), ("heads", ctypes.c_int32), ("row_bytes", ctypes.c_int32),
+                ("fill", ctypes.c_uint32)]
+
+
 class SasError(RuntimeError):
     def __init__(self, status, message):
         super().__init__(f"{message} (status {status})")
@@ -87,6 +92,8 @@ def lib():
     L.sas_attention_fwd.restype = i32
     L.sas_attention_fwd_noisy.argtypes = [vp] * 13
     L.sas_attention_fwd_noisy.restype = i32
+    L.sas_fill_varlen_tails.argtypes = [vp, ctypes.POINTER(SasTail), i32, vp]
+    L.sas_fill_varlen_tails.restype = i32
     L.sas_attention_fwd_varlen.argtypes = [vp, vp, i32] + [vp] * 11
     L.sas_attention_fwd_varlen.restype = i32
     L.sas_attention_bwd.argtypes = [vp] * 16
@@ -219,6 +226,13 @@ def sas_attention_fwd_varlen(h, cu_seqlens, Q, K, V, scores, O, LSE=None, sel_id
     _check(st, h, "sas_attention_fwd_varlen")
 
 
+def sas_fill_varlen_tails(h, tails, stream=None):
+    """tails: (contiguous tensor of heads x N rows, heads, bytes per row, 32-bit fill word)."""
+    arr = (SasTail * len(tails))(*(SasTail(x.data_ptr(), heads, width, fill & 0xffffffff)
+                                   for x, heads, width, fill in tails))
+    _check(lib().sas_fill_varlen_tails(h, arr, len(tails), _stream(stream)), h, "sas_fill_varlen_tails")
+
+
 def sas_attention_fwd(h, Q, K, V, O, scores=None, Wq=None, Wk=None, LSE=None, sel_idx=None, sel_logg=None,
                       stream=None):
     bf = torch.bfloat16
@@ -344,6 +358,7 @@ class SasLayer:
                  scope=SAS_SCOPE_SPARSE):
         self.B, self.H, self.N, self.d, self.topk = B, H, N, d, topk
         self.mode = mode
+        self.max_len = max_seqlen or N           # of one sequence
         self.Hkv = Hkv or H                      # kept lists are per KV group
         self.selector = selector
         self.scope = scope
@@ -354,18 +369,34 @@ class SasLayer:
                          Wk=None):
         """Packed sequences (handle made with max_seqs > 0): Q [H, N, d], K/V [Hkv, N, d],
         scores [Hkv, N, C] (or the learned selector's Wq, Wk), cu_seqlens int32 on the
-        device.  The library does not write rows past cu[-1]: they keep the fill of
-        the tensors made here (0, and sel_fill in sel_idx)."""
+        device.  The forward does not write rows past cu[-1]: they are filled here
+        (0, and sel_fill in sel_idx)."""
         dev = Q.device
-        O = torch.zeros_like(Q)
-        LSE = torch.zeros(self.H, self.N, device=dev, dtype=torch.float32)
+        tails = []
+        O = self._packed_like(Q, self.H, tails)
+        LSE = torch.empty(self.H, self.N, device=dev, dtype=torch.float32)
+        tails.append((LSE, self.H, 4, 0))
         sel_idx = sel_logg = None
-        if want_sel:
+        if want_sel and self.topk > 0 and self.scope == SAS_SCOPE_SPARSE:
+            sel_idx = torch.empty(self.Hkv, self.N, self.topk, device=dev, dtype=torch.int32)
+            sel_logg = torch.empty(self.Hkv, self.N, self.topk, device=dev, dtype=torch.float32)
+            tails += [(sel_idx, self.Hkv, 4 * self.topk, sel_fill), (sel_logg, self.Hkv, 4 * self.topk, 0)]
+        elif want_sel:
             k = max(self.topk, 1)
             sel_idx = torch.full((self.Hkv, self.N, k), sel_fill, device=dev, dtype=torch.int32)
             sel_logg = torch.zeros(self.Hkv, self.N, k, device=dev, dtype=torch.float32)
         sas_attention_fwd_varlen(self.h, cu_seqlens, Q, K, V, scores, O, LSE, sel_idx, sel_logg, stream, Wq, Wk)
+        if tails:
+            sas_fill_varlen_tails(self.h, tails, stream)
         return O, LSE, sel_idx, sel_logg
+
+    def _packed_like(self, x, heads, tails):
+        """A tensor like x for the kernels to fill, its spare rows noted in tails."""
+        if x.numel() != heads * self.N * self.d:
+            return torch.zeros_like(x)
+        out = torch.empty_like(x)
+        tails.append((out, heads, self.d * x.element_size(), 0))
+        return out
 
     def _outputs(self, Q, want_sel):
         dev = Q.device
@@ -409,14 +440,27 @@ class SasLayer:
                              stream=None):
         """Backward of the last attention_varlen on this handle: Q, O, dO [H, N, d],
         K, V [Hkv, N, d].  Returns (dQ, dK, dV, dlogg [Hkv, N, topk], dscores [Hkv, N, C]
-        or None); rows past cu[-1] keep the zero fill of the tensors made here."""
+        or None); rows past cu[-1] are zero."""
         dev = Q.device
-        dQ, dK, dV = torch.zeros_like(Q), torch.zeros_like(K), torch.zeros_like(V)
-        dlogg = torch.zeros(self.Hkv, self.N, max(self.topk, 1), device=dev, dtype=torch.float32)
+        tails = []
+        dQ = self._packed_like(Q, self.H, tails)
+        dK, dV = self._packed_like(K, self.Hkv, tails), self._packed_like(V, self.Hkv, tails)
+        if self.topk > 0 and self.scope == SAS_SCOPE_SPARSE:
+            dlogg = torch.empty(self.Hkv, self.N, self.topk, device=dev, dtype=torch.float32)
+            tails.append((dlogg, self.Hkv, 4 * self.topk, 0))
+        else:
+            dlogg = torch.zeros(self.Hkv, self.N, max(self.topk, 1), device=dev, dtype=torch.float32)
         ds = None
         if want_ds:
-            ds = torch.zeros(self.Hkv, self.N, scores.shape[-1], device=dev, dtype=torch.float32)
+            shape = (self.Hkv, self.N, scores.shape[-1])
+            if shape[-1] == -(-self.max_len // 64):
+                ds = torch.empty(shape, device=dev, dtype=torch.float32)
+                tails.append((ds, self.Hkv, 4 * shape[-1], 0))
+            else:
+                ds = torch.zeros(shape, device=dev, dtype=torch.float32)
         sas_attention_bwd(self.h, Q, K, V, O, LSE, dO, dQ, dK, dV, scores, sel_idx, sel_logg, dlogg, ds, stream)
+        if tails:
+            sas_fill_varlen_tails(self.h, tails, stream)
         return dQ, dK, dV, dlogg, ds
 
     def mlp(self, X, W1, W2, b1=None, b2=None, stream=None):
