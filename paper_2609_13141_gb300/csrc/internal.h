@@ -192,8 +192,8 @@ struct DecodeArgs {
     int cluster;                // 1: a group's attention CTAs form one cluster and merge among themselves
 };
 constexpr int kDecScoreChunk = 256;
-// Attention split for `groups` lists of at most max_len entries on sms SMs.
-void decode_attn_split(int max_len, int d, bool dense, int groups, int sms, int* nsplit, int* bpc, int* nst,
+// Attention split for `groups` lists of at most max_len entries, G query heads each, on sms SMs.
+void decode_attn_split(int max_len, int d, bool dense, int groups, int G, int sms, int* nsplit, int* bpc, int* nst,
                        int* cluster);
 // Dynamic shared memory the score and attention kernels need.
 size_t decode_score_smem(int nsplit, int topk, int d_sel);

@@ -41,7 +41,9 @@ constexpr int kPrepThreads = 256;
 constexpr int kScoreThreads = 256;
 constexpr int kAttnThreads = 256;
 constexpr int kStages = 3;
-constexpr int kRankMax = 512;         // candidates ranked by counting (M^2 comparisons); more take the radix select
+constexpr int kRankRows = 96;         // blocks of a score CTA ranked by counting; more are sorted (score kernel, us,
+                                      // counting / sorting: 76 blocks 4.2 / 4.5, 129 6.4 / 5.5, 256 and 221 8.0 / 6.2)
+constexpr int kRankMax = 256;         // candidates ranked by counting, one a thread; more take the radix select
 constexpr float kLog2e = 1.4426950408889634f;
 
 __device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
@@ -289,6 +291,31 @@ __device__ __forceinline__ uint32_t order_key(float f) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
+// Descending bitonic sort of 256 distinct 64-bit keys, one per thread of the
+// CTA; returns the key that ends at position threadIdx.x.  Exchanges within a
+// warp use shuffles, wider ones the 256-entry shared buffer xchg.
+__device__ uint64_t bitonic256_desc(uint64_t c, uint64_t* xchg) {
+    const int t = threadIdx.x;
+#pragma unroll
+    for (int k = 2; k <= 256; k <<= 1) {
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            uint64_t o;
+            if (j >= 32) {
+                xchg[t] = c;
+                __syncthreads();
+                o = xchg[t ^ j];
+                __syncthreads();
+            } else {
+                o = __shfl_xor_sync(0xffffffffu, c, j);
+            }
+            const bool keep_max = ((t & j) == 0) == ((t & k) == 0);
+            c = keep_max ? (c > o ? c : o) : (c < o ? c : o);
+        }
+    }
+    return c;
+}
+
 // How many of the M keys (16-byte aligned, the rest of the last four slots 0) rank
 // ahead of key (>= 1) at position t: the larger ones, and the equal ones listed
 // before it.  All lanes of a warp read the same four keys at a time; the
@@ -308,31 +335,24 @@ __device__ __forceinline__ int rank_of(const uint32_t* keys, int M, uint32_t key
     return r;
 }
 
-// Exact Top-K of at most 512 candidates in ascending block order by counting each
-// one's rank (M^2 comparisons, about 1 us at 160 candidates, against 4 us of the
-// radix select's three histogram passes); same arguments as select_candidates.
-__device__ void select_by_rank(const DecodeArgs& a, int bh, int M, const uint32_t* keys, const int32_t* idx,
+// Exact Top-K of at most kRankMax candidates in ascending block order by counting
+// each one's rank (M^2 comparisons, about 1 us at 160 candidates, against 4 us of the
+// radix select's three histogram passes; two candidates a thread lose: one sequence of
+// 205325 tokens, 416 candidates: 28.2 us against 17.5 for the radix select); same arguments as select_candidates.
+__device__ __forceinline__ void select_by_rank(const DecodeArgs& a, int bh, int M, const uint32_t* keys, const int32_t* idx,
                                int* scan) {
     const int K = a.topk, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     int32_t* lst = a.list + static_cast<size_t>(bh) * 64;
     int32_t* so = a.sel_idx ? a.sel_idx + static_cast<size_t>(bh) * K : nullptr;
-    bool take[2];
-    unsigned bal[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int i = h * kScoreThreads + t;
-        const uint32_t k = i < M ? keys[i] : 0u;
-        take[h] = k != 0 && rank_of(keys, M, k, i, i - lane) < K;
-        bal[h] = __ballot_sync(0xffffffffu, take[h]);
-        if (lane == 0) scan[h * 8 + warp] = __popc(bal[h]);
-    }
+    const uint32_t k = t < M ? keys[t] : 0u;
+    const bool take = k != 0 && rank_of(keys, M, k, t, t - lane) < K;
+    const unsigned bal = __ballot_sync(0xffffffffu, take);
+    if (lane == 0) scan[warp] = __popc(bal);
     __syncthreads();
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        if (!take[h]) continue;
-        int pos = __popc(bal[h] & ((1u << lane) - 1u));
-        for (int w = 0; w < h * 8 + warp; ++w) pos += scan[w];
-        const int m = idx[h * kScoreThreads + t];
+    if (take) {
+        int pos = __popc(bal & ((1u << lane) - 1u));
+        for (int w = 0; w < warp; ++w) pos += scan[w];
+        const int m = idx[t];
         lst[pos] = m;
         if (so) so[pos] = m;
     }
@@ -343,7 +363,7 @@ __device__ void select_by_rank(const DecodeArgs& a, int bh, int M, const uint32_
 // order, ties to the lower block: radix select of the K-th largest key tau in
 // digits of 12, 10 and 10 bits, then every key > tau plus the first keys == tau,
 // emitted in list order.  256 threads; K < number of non-empty candidates.
-__device__ void select_candidates(const DecodeArgs& a, int bh, int M, const uint32_t* keys, const int32_t* idx,
+__device__ __forceinline__ void select_candidates(const DecodeArgs& a, int bh, int M, const uint32_t* keys, const int32_t* idx,
                                   int* hist, int* scan, int* bc) {
     const int K = a.topk;
     const int t = threadIdx.x, lane = t & 31;
@@ -508,10 +528,20 @@ __global__ void __launch_bounds__(kScoreThreads) dec_score_kernel(DecodeArgs a, 
         }
         // local Top-K of this CTA's blocks: those with fewer than K ahead of them
         bool take = t < rows_cta && key != 0;
-        if (rows_cta > K) {
+        if (rows_cta > K && rows_cta <= kRankRows) {
             xchg[t] = take ? key : 0u;
             __syncthreads();
             take = take && rank_of(xchg, (rows_cta + 3) & ~3, key, t, warp * 32) < K;
+        } else if (rows_cta > K) {
+            // sort the distinct keys (score key, then the lower block first) and keep
+            // those at or above the K-th
+            uint64_t* sx = reinterpret_cast<uint64_t*>(smem + L.hist);
+            const uint64_t comp = (static_cast<uint64_t>(key) << 32) | (0xffffffffu - static_cast<uint32_t>(t));
+            const uint64_t sorted = bitonic256_desc(comp, sx);
+            __syncthreads();
+            if (t == K - 1) sx[0] = sorted;
+            __syncthreads();
+            take = take && comp >= sx[0];
         }
         // compact the kept blocks in block order into this CTA's K candidate slots
         const unsigned bal = __ballot_sync(0xffffffffu, take);
@@ -998,8 +1028,6 @@ __global__ void __launch_bounds__(kTcThreads) dec_attn_tc_kernel(const __grid_co
     const int n = __ldg(a.seq_lens + b);
     const bool bad = bad_len(n, a);   // recorded by the prep kernel
     const int c = bad ? 0 : (n - 1) / kBlk;
-    const int j0 = blockIdx.x * a.bpc;
-
 #define SAS_TC_LOAD(e) tc_load_page(smem, nst, ent, (e), &mapK, &mapV, full, a.Hkv, g)
 
     // --- set-up that needs nothing from the preceding kernel
@@ -1013,7 +1041,7 @@ __global__ void __launch_bounds__(kTcThreads) dec_attn_tc_kernel(const __grid_co
         // the current block (entry 0) was appended by the prep kernel, which the
         // score kernel waited for before letting this grid start, so its page can
         // load now (dense mode: the prep kernel precedes this one directly)
-        if (!bad && j0 == 0 && !a.dense) {
+        if (!bad && blockIdx.x == 0 && !a.dense) {
             int page = __ldg(a.block_table + static_cast<size_t>(b) * a.max_blocks + c);
             if (page < 0 || page >= a.num_pages) page = -1;   // recorded by the prep kernel
             ent[0] = c;
@@ -1037,8 +1065,11 @@ __global__ void __launch_bounds__(kTcThreads) dec_attn_tc_kernel(const __grid_co
     }
     grid_dep_wait();   // the kept list
     const int L = bad ? 0 : (a.dense ? c : __ldg(a.list_n + bh)) + 1;
-    const int cnt = bad ? 0 : max(0, min(j0 + a.bpc, L) - j0);
-    const int first = (j0 == 0 && !a.dense) ? 1 : 0;   // entries set up before the wait
+    // a cluster shares its list's pages evenly (a short history has fewer than bpc a CTA)
+    const int per = a.cluster ? (L + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x) : a.bpc;
+    const int j0 = blockIdx.x * per;
+    const int cnt = bad ? 0 : max(0, min(j0 + per, L) - j0);
+    const int first = (blockIdx.x == 0 && !a.dense) ? 1 : 0;   // entries set up before the wait
     for (int jj = first + t; jj < cnt; jj += kTcThreads) {
         const int j = j0 + jj;
         const int blk = j == 0 ? c : (a.dense ? j - 1 : __ldg(a.list + static_cast<size_t>(bh) * 64 + j - 1));
@@ -1282,7 +1313,7 @@ __global__ void __launch_bounds__(kTcThreads) dec_attn_tc_kernel(const __grid_co
     if (bad) return;
 
     // merge the partials of the splits the list reached
-    const int used = (L + a.bpc - 1) / a.bpc;
+    const int used = (L + per - 1) / per;
     const float* pgp = a.part + static_cast<size_t>(bh) * a.nsplit_a * G * (D + 2);
     float* mw = reinterpret_cast<float*>(smem);    // [used][G][2], in the free stage
     for (int i = t; i < used * G; i += kTcThreads) {
@@ -1437,25 +1468,62 @@ cudaError_t launch_score_d(const DecodeArgs& a, const KernelEnv& env) {
 
 }  // namespace
 
-void decode_attn_split(int max_len, int d, bool dense, int groups, int sms, int* nsplit, int* bpc, int* nst,
+namespace {
+
+// Clusters of S attention CTAs (a ring of nst stages, bpc pages each) that the device
+// holds at once; 0 if it cannot say.
+int attn_clusters_at_once(int S, int nst, int bpc, int G) {
+    const void* f = G == 1   ? reinterpret_cast<const void*>(dec_attn_tc_kernel<1>)
+                    : G == 2 ? reinterpret_cast<const void*>(dec_attn_tc_kernel<2>)
+                    : G == 4 ? reinterpret_cast<const void*>(dec_attn_tc_kernel<4>)
+                             : reinterpret_cast<const void*>(dec_attn_tc_kernel<8>);
+    const size_t smem = tc_layout(nst, bpc).total;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim = {static_cast<unsigned>(S), 1, 1};
+    cfg.gridDim = dim3(static_cast<unsigned>(S));
+    cfg.blockDim = dim3(kTcThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (ensure_smem_attr(f, smem, false, true) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, f, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return n;
+}
+
+}  // namespace
+
+void decode_attn_split(int max_len, int d, bool dense, int groups, int G, int sms, int* nsplit, int* bpc, int* nst,
                        int* cluster) {
     int per;
     *cluster = 0;
     if (d == 128 && !dense) {
+
         // tensor-core kernel, a SAS list (at most 65 pages): a cluster of S <= 16 CTAs
         // per group, as many as run at once, merging over distributed shared memory.
         // Three CTAs of one 64 KB stage share an SM, but whole clusters have to find
         // room in a GPC, so the grid stays at 8/3 of the SMs (64 groups of 33 pages:
-        // 28.8, 25.7, 23.6, 20.8 and 32.0 us with S = 3, 4, 5, 6 and 7).  One CTA per
-        // SM or fewer: up to three stages, so that a CTA's own loads overlap.  (Before:
-        // one page pair per CTA and a merge through global memory by the last one to
-        // arrive; 64 groups took 2.4 waves and 36.5 us.)
+        // 28.8, 25.7, 23.6, 20.8 and 32.0 us with S = 3, 4, 5, 6 and 7; the device's own
+        // count of clusters that fit stops earlier, 45.4 us a step for 39.8).  One
+        // CTA per SM or fewer: up to three stages, so that a CTA's own loads overlap, and
+        // there the device's count decides (8 groups of 49 pages: thirteen CTAs each do
+        // not all find room and take 19.5 us, two waves).  (Before: one page pair per CTA
+        // and a merge through global memory by the last one to arrive; 64 groups took 2.4
+        // waves and 36.5 us.)
         const int fit = 8 * sms / (3 * (groups > 0 ? groups : 1));
         int S = fit < 1 ? 1 : (fit > kMaxDecCluster ? kMaxDecCluster : fit);
-        per = (max_len + S - 1) / S;
-        S = (max_len + per - 1) / per;
-        const int steps = (per + 1) / 2;
-        *nst = static_cast<long long>(groups) * S <= sms ? (steps < 3 ? steps : 3) : 1;
+        for (;; --S) {
+            per = (max_len + S - 1) / S;
+            S = (max_len + per - 1) / per;
+            const int steps = (per + 1) / 2;
+            const bool spread = static_cast<long long>(groups) * S <= sms;
+            *nst = spread ? (steps < 3 ? steps : 3) : 1;
+            if (S == 1 || !spread || attn_clusters_at_once(S, *nst, per, G) >= groups) break;
+        }
         *cluster = 1;
     } else if (d == 128) {
         // dense lists: cut into at most 64 (128 past 2048 pages) pieces of whole
