@@ -349,6 +349,8 @@ __device__ __forceinline__ void select_by_rank(const DecodeArgs& a, int bh, int 
     const unsigned bal = __ballot_sync(0xffffffffu, take);
     if (lane == 0) scan[warp] = __popc(bal);
     __syncthreads();
+    int total = 0;   // K, or fewer when a summary load gave up and left candidates empty
+    for (int w = 0; w < kScoreThreads / 32; ++w) total += scan[w];
     if (take) {
         int pos = __popc(bal & ((1u << lane) - 1u));
         for (int w = 0; w < warp; ++w) pos += scan[w];
@@ -356,13 +358,16 @@ __device__ __forceinline__ void select_by_rank(const DecodeArgs& a, int bh, int 
         lst[pos] = m;
         if (so) so[pos] = m;
     }
-    if (t == 0) a.list_n[bh] = K;
+    if (so)
+        for (int e = total + t; e < K; e += kScoreThreads) so[e] = -1;
+    if (t == 0) a.list_n[bh] = total;
 }
 
 // Exact Top-K of M candidates (keys[i], block idx[i]) listed in ascending block
 // order, ties to the lower block: radix select of the K-th largest key tau in
 // digits of 12, 10 and 10 bits, then every key > tau plus the first keys == tau,
-// emitted in list order.  256 threads; K < number of non-empty candidates.
+// emitted in list order.  256 threads; K <= M.  Empty candidates (key 0) are never
+// kept: with fewer than K others (a summary load that gave up) the list is shorter.
 __device__ __forceinline__ void select_candidates(const DecodeArgs& a, int bh, int M, const uint32_t* keys, const int32_t* idx,
                                   int* hist, int* scan, int* bc) {
     const int K = a.topk;
@@ -415,6 +420,7 @@ __device__ __forceinline__ void select_candidates(const DecodeArgs& a, int bh, i
         r = bc[1];
     }
     const uint32_t tau = prefix;   // the K-th largest key; take the first r keys equal to it
+    if (tau == 0) r = 0;
     // list-order emission: contiguous ranges of odd length per thread (conflict-free reads)
     const int per = ((M + kScoreThreads - 1) / kScoreThreads) | 1;
     const int lo = min(t * per, M), hi = min(lo + per, M);
@@ -446,7 +452,11 @@ __device__ __forceinline__ void select_candidates(const DecodeArgs& a, int bh, i
             ++pos;
         }
     }
-    if (t == 0) a.list_n[bh] = K;
+    if (t == kScoreThreads - 1) {   // the last range ends the list
+        a.list_n[bh] = pos;
+        if (so)
+            for (int e = pos; e < K; ++e) so[e] = -1;
+    }
 }
 
 // grid (nsplit_s, B*Hkv), launched as a programmatic dependent of the prep kernel.
@@ -601,13 +611,15 @@ __global__ void __launch_bounds__(kScoreThreads) dec_score_kernel(DecodeArgs a, 
     }
     const size_t gbase = static_cast<size_t>(bh) * a.nsplit_s * Kc;
     if (C <= kDecScoreChunk) {
-        // one CTA held every block: its local Top-K is the group's, already in block order
-        for (int e = t; e < K; e += kScoreThreads) {
-            const int m = alone ? my_idx[e] : __ldcg(a.cand_idx + gbase + e);
-            lst[e] = m;
-            if (so) so[e] = m;
+        // one CTA held every block: its local Top-K is the group's, already in block
+        // order (-1 past the blocks whose summaries arrived; K <= 64 < 256 threads)
+        const int m = t < K ? (alone ? my_idx[t] : __ldcg(a.cand_idx + gbase + t)) : -1;
+        if (t < K) {
+            lst[t] = m;
+            if (so) so[t] = m;
         }
-        if (t == 0) a.list_n[bh] = K;
+        const int kept = __syncthreads_count(m >= 0);
+        if (t == 0) a.list_n[bh] = kept;
         return;
     }
     const int M = ((C + kDecScoreChunk - 1) / kDecScoreChunk) * Kc;   // the splits that held blocks
@@ -628,6 +640,16 @@ __global__ void __launch_bounds__(kScoreThreads) dec_score_kernel(DecodeArgs a, 
 }
 
 // ---------------------------------------------------------------- attention
+
+// Page of block blk of sequence b, whose own block is c.  -1, and nothing is read, for a
+// block it does not have; -1 and the status word for a table entry outside the cache.
+__device__ __forceinline__ int block_page(const DecodeArgs& a, int b, int blk, int c, int* status) {
+    if (static_cast<unsigned>(blk) > static_cast<unsigned>(c)) return -1;
+    const int page = __ldg(a.block_table + static_cast<size_t>(b) * a.max_blocks + blk);
+    if (page >= 0 && page < a.num_pages) return page;
+    atomicExch(status, kStatusBadInput);
+    return -1;
+}
 
 // Shared-memory layout of the attention kernel for a ring of nst stages.
 struct AttnLayout {
@@ -713,13 +735,8 @@ __global__ void __launch_bounds__(kAttnThreads) dec_attn_kernel(DecodeArgs a, in
     for (int jj = first + t; jj < cnt; jj += kAttnThreads) {
         const int j = j0 + jj;
         const int blk = j == 0 ? c : (a.dense ? j - 1 : __ldg(a.list + static_cast<size_t>(bh) * 64 + j - 1));
-        int page = __ldg(a.block_table + static_cast<size_t>(b) * a.max_blocks + blk);
-        if (page < 0 || page >= a.num_pages) {
-            atomicExch(status, kStatusBadInput);
-            page = -1;
-        }
         ent[2 * jj] = blk;
-        ent[2 * jj + 1] = page;
+        ent[2 * jj + 1] = block_page(a, b, blk, c, status);
     }
     __syncthreads();
     int issued = first;
@@ -1073,13 +1090,8 @@ __global__ void __launch_bounds__(kTcThreads) dec_attn_tc_kernel(const __grid_co
     for (int jj = first + t; jj < cnt; jj += kTcThreads) {
         const int j = j0 + jj;
         const int blk = j == 0 ? c : (a.dense ? j - 1 : __ldg(a.list + static_cast<size_t>(bh) * 64 + j - 1));
-        int page = __ldg(a.block_table + static_cast<size_t>(b) * a.max_blocks + blk);
-        if (page < 0 || page >= a.num_pages) {
-            atomicExch(status, kStatusBadInput);
-            page = -1;
-        }
         ent[2 * jj] = blk;
-        ent[2 * jj + 1] = page;
+        ent[2 * jj + 1] = block_page(a, b, blk, c, status);
     }
     fence_proxy_async_smem();   // Q and P writes before the tensor cores read them
     tc_fence_before();
