@@ -176,6 +176,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         uint32_t ph = 0;
         int it = 0;
         bool ok = true;
+        // no bounded wait runs while the kernel that writes A does: its time is not this one's
+        if (p.early_b) pdl_wait();
         for (int t = blockIdx.x; t < total && ok; t += gridDim.x, ++it) {
             const int acc = it & 1;
             const uint32_t aph = (it >> 1) & 1;
@@ -349,7 +351,9 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constan
         for (int q = issued - 1; q >= 0 && q >= issued - Cfg::STAGES; --q)
             mbar_wait_drain(&full_bar[q % Cfg::STAGES], (q / Cfg::STAGES) & 1, p.limit, p.status);
     } else if (warp == 1) {
-        // ---------------- MMA issuer (whole warp; the elected lane issues)
+        // ---------------- MMA issuer (whole warp; the elected lane issues).  The wait for
+        // the kernel that writes A comes first: its time is not on the bounded waits' budget
+        if (p.early_b) pdl_wait();
         for (int kb = 0; kb < nk; ++kb) {
             const int s = kb % Cfg::STAGES;
             if (!mbar_wait_warp(&full_bar[s], (kb / Cfg::STAGES) & 1, wc, kSuspendNs)) break;
