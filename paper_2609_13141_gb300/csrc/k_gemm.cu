@@ -19,6 +19,8 @@
 // Problems whose tiles do not fill the chip take gemm_split_kernel: a cluster
 // of CTAs splits one tile's K and adds the partial sums over distributed
 // shared memory.  pick_shape() chooses between the two and their tile widths.
+#include <mutex>
+
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -473,6 +475,49 @@ cudaError_t launch_ex(void (*kernel)(Params...), int grid, int smem, int cluster
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Clusters of s split CTAs of 128 x BN tiles for which the device has room at one CTA
+// an SM (a cluster has to find it in one GPC); 0 if it cannot say.
+template <int BN>
+int split_clusters(int s) {
+    using Cfg = SplitCfg<BN>;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(s);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = Cfg::SMEM;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim = {static_cast<unsigned>(s), 1, 1};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (ensure_smem_attr(reinterpret_cast<const void*>(gemm_split_kernel<BN>), Cfg::SMEM) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, gemm_split_kernel<BN>, &cfg) == cudaSuccess)
+        return n;
+    cudaGetLastError();
+    return 0;
+}
+
+// SMs of the current device and those counts, asked for by its first problem.
+struct Room {
+    int sms, bn128[kMaxSplit + 1], bn64[kMaxSplit + 1];
+};
+const Room& device_room() {
+    constexpr int kMaxDevices = 128;
+    static Room rooms[kMaxDevices + 1];   // the last: no device known, one SM and no cluster
+    static std::once_flag once[kMaxDevices + 1];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) dev = kMaxDevices;
+    Room& r = rooms[dev];
+    std::call_once(once[dev], [&r, dev] {
+        r.sms = dev < kMaxDevices ? device_sm_count() : 1;
+        for (int s = 2; s <= kMaxSplit && dev < kMaxDevices; ++s) {
+            r.bn128[s] = split_clusters<128>(s);
+            r.bn64[s] = 2 * split_clusters<64>(s);   // two share an SM, which the count leaves out
+        }
+    });
+    return r;
+}
+
 template <int BN>
 cudaError_t launch_split(const GemmProblem& p, int split, const KernelEnv& env, const char** err) {
     using Cfg = SplitCfg<BN>;
@@ -518,16 +563,20 @@ cudaError_t launch_bn(const GemmProblem& p, const KernelEnv& env, const char** e
 // BN = 256, 128, 64 (tensor time 512, 256 and 192; the operand bytes an SM takes
 // from L2, 48, 32 and 24 KB, hold the narrow tiles); tiles go in whole waves.
 // A split tile's CTAs run together (BN = 64: two per SM share it) and pay the
-// exchange of partial sums, about 3000 cycles.  Measured (us for both MLP
+// exchange of partial sums, about 3000 cycles.  A split is taken only where the device
+// holds all its clusters at once: with 48 clusters of three where 46 find room, 1024
+// rows of 768 x 3072 took 38 us, with 48 pairs 29 (64 rows of 2560 x 9728: 42 and 31,
+// 500 rows of 1536 x 6144: 50 and 38).  Measured (us for both MLP
 // products, 256-wide tiles on one CTA per tile -> this choice): 2560 x 9728 at
-// 64 rows 86 -> 45, 256 rows 86 -> 47, 777 rows 110 -> 90 (its down-projection
+// 64 rows 84 -> 31, 256 rows 87 -> 46, 777 rows 103 -> 85 (its down-projection
 // has 70 tiles of 256 columns for 152 SMs, 140 of 128); 1024 x 4096 at 64 rows
-// 39 -> 22.  With the narrow tiles' tensor time alone in the estimate, 4096 rows
+// 41 -> 19.  With the narrow tiles' tensor time alone in the estimate, 4096 rows
 // of 3072 x 12288 took 128-wide tiles and went from 421 to 499.
 struct GemmShape {
     int bn, split;
 };
-GemmShape pick_shape(int M, int N, int K, int sms) {
+GemmShape pick_shape(int M, int N, int K, const Room& room) {
+    const int sms = room.sms;
     const long long mt = (M + kBM - 1) / kBM, kb = K / kBK;
     GemmShape best{64, 0};
     long long cost = -1;
@@ -545,7 +594,7 @@ GemmShape pick_shape(int M, int N, int K, int sms) {
             if (tiles * s > slots || kb < 4 * s) continue;
             const long long both = tiles * s > sms ? 2 : 1;   // CTAs on the fullest SM
             const long long cs = (kb + s - 1) / s * per * both + 3000;
-            if (cs < cost) {
+            if (cs < cost && tiles <= (bn == 128 ? room.bn128[s] : room.bn64[s])) {
                 cost = cs;
                 best = {bn, s};
             }
@@ -557,7 +606,7 @@ GemmShape pick_shape(int M, int N, int K, int sms) {
 }  // namespace
 
 cudaError_t launch_gemm(const GemmProblem& p, const KernelEnv& env, const char** err) {
-    const GemmShape g = p.batches == 1 && p.ldc == p.N ? pick_shape(p.M, p.N, p.K, device_sm_count()) : GemmShape{p.N % 256 == 0 ? 256 : (p.N % 128 == 0 ? 128 : 64), 0};
+    const GemmShape g = p.batches == 1 && p.ldc == p.N ? pick_shape(p.M, p.N, p.K, device_room()) : GemmShape{p.N % 256 == 0 ? 256 : (p.N % 128 == 0 ? 128 : 64), 0};
     if (g.split > 0) return g.bn == 128 ? launch_split<128>(p, g.split, env, err) : launch_split<64>(p, g.split, env, err);
     switch (g.bn) {
         case 256: return launch_bn<256>(p, env, err);
