@@ -1744,26 +1744,25 @@ cudaError_t launch_varlen_tiles(const int32_t* cu, int S, int Ncap, int max_len,
 
 namespace {
 
-// CTA (x, y) fills part x of head y's spare rows in each tensor.  Mostly there are
+// CTA (x, y) fills part x of the spare rows of heads y, y + grid.y, ... in each tensor.  Mostly there are
 // few: clearing whole outputs ahead of the kernels that write nearly all of them
 // again took 49 us of the 710 of a 32-head call over 19000 packed tokens (155 MB of
 // O alone), this 2 us.
 __global__ void __launch_bounds__(256) varlen_tails_kernel(TailFill f, int N, const int* ntiles) {
     const int first = min(max(__ldg(ntiles + 1), 0), N);
-    const int head = blockIdx.y;
     if (first >= N) return;
+    const long long start = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const long long step = static_cast<long long>(gridDim.x) * blockDim.x;
     for (int k = 0; k < f.count; ++k) {
-        if (head >= f.heads[k]) continue;
-        const long long w = f.row_words[k];
-        uint32_t* p = f.ptr[k] + (static_cast<long long>(head) * N + first) * w;
-        const long long n = (N - first) * w;
+        const long long w = f.row_words[k], n = (N - first) * w;
         const uint32_t v = f.fill[k];
-        const long long start = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-        const long long step = static_cast<long long>(gridDim.x) * blockDim.x;
-        if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0 && n % 4 == 0) {
-            for (long long i = start; i < n / 4; i += step) reinterpret_cast<uint4*>(p)[i] = make_uint4(v, v, v, v);
-        } else {
-            for (long long i = start; i < n; i += step) p[i] = v;
+        for (long long head = blockIdx.y; head < f.heads[k]; head += gridDim.y) {
+            uint32_t* p = f.ptr[k] + (head * N + first) * w;
+            if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0 && n % 4 == 0) {
+                for (long long i = start; i < n / 4; i += step) reinterpret_cast<uint4*>(p)[i] = make_uint4(v, v, v, v);
+            } else {
+                for (long long i = start; i < n; i += step) p[i] = v;
+            }
         }
     }
 }
@@ -1773,7 +1772,7 @@ __global__ void __launch_bounds__(256) varlen_tails_kernel(TailFill f, int N, co
 cudaError_t launch_varlen_tails(const TailFill& f, int N, const int* ntiles, const KernelEnv& env) {
     int heads = 1;
     for (int k = 0; k < f.count; ++k) heads = max(heads, f.heads[k]);
-    varlen_tails_kernel<<<dim3(8, heads), 256, 0, env.stream>>>(f, N, ntiles);
+    varlen_tails_kernel<<<dim3(8, min(heads, 65535)), 256, 0, env.stream>>>(f, N, ntiles);
     return cudaGetLastError();
 }
 

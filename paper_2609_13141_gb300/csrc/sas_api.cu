@@ -610,8 +610,8 @@ sas_status sas_fill_varlen_tails(sas_handle* h, const sas_tail* tails, int32_t c
     sas::TailFill f{};
     for (int32_t k = 0; k < count; ++k) {
         const sas_tail& t = tails[k];
-        if (!t.ptr || !aligned4(t.ptr) || t.row_bytes < 4 || t.row_bytes % 4 != 0 || t.heads < 1 || t.heads > 65535)
-            return fail(h, SAS_ERR_INVALID_ARG, "tails: 4-byte aligned rows of whole words, 1 .. 65535 heads");
+        if (!t.ptr || !aligned4(t.ptr) || t.row_bytes < 4 || t.row_bytes % 4 != 0 || t.heads < 1)
+            return fail(h, SAS_ERR_INVALID_ARG, "tails: 4-byte aligned rows of whole words, at least one head");
         f.ptr[k] = static_cast<uint32_t*>(t.ptr);
         f.heads[k] = t.heads;
         f.row_words[k] = t.row_bytes / 4;
