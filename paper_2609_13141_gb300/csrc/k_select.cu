@@ -541,22 +541,31 @@ __global__ void __launch_bounds__(128, 3) select_given_kernel(SelParams p) {
 // The rows come to shared memory by coalesced asynchronous copies and every pass
 // over them is a short loop, so the work does not depend on how neighbouring rows'
 // selections differ, and what a row costs whatever its length (reductions, bracket
-// updates, addresses) is shared by four.  The K-th largest score is bracketed: a
-// first guess from the mean and deviation of the row's first 128 scores (a normal
-// sample's K-th largest), one Newton step, then interpolation on the counts with a
-// midpoint every third step, and past kValueSteps counts bisection of the float
-// order, which ends at a value shared by the boundary blocks: ties then go to the
-// lower blocks.  NaN ranks as replace-the-worst has it: one among the first K blocks
-// stays, a later one never enters.
-// At 8 groups x 32768 rows, K = 32 (268 MB of scores, 40 us at the copy rate): 207 us,
-// 640 instructions a row, 70% of the issue slots; a thread per row and the segments'
-// lists in a launch of their own took 343 + 58.
+// updates, addresses) is shared by four.  The K-th largest score is bracketed by
+// scores of the row: a pass counts the scores at or above a threshold and finds the
+// next score on the side that matters, so a bracket that holds one value only ends the
+// search (ties then go to the lower blocks), as does one that misses K by one.  The
+// first threshold comes from the mean and deviation of the row's first 128 scores (a
+// normal sample's K-th largest), those more than kFar below the maximum, masked blocks
+// among them, left out; then Newton, interpolation on the counts, and from the fourth
+// pass on interpolation and every third time a midpoint in the float order, which suits
+// scores over many magnitudes and bounds the search.  NaN ranks as replace-the-worst
+// has it: one among the first K blocks stays, a later one never enters.
+// At 8 groups x 32768 rows, K = 32 (268 MB of scores, 40 us at the copy rate): 194 us,
+// most of it instruction issue; a thread per row and the segments' lists in a launch
+// of their own took 408.  24 heads x 2 x 6001 rows, K = 16, normal scores / half the
+// blocks masked / rounded to halves: 58 / 56 / 52 us (77 / 64 / 75 with a thread per
+// row; 68 / 120 / 172 when the search closed in on the values alone, from a mean and
+// deviation over every score).  The slowest of four rows takes 3 passes on these, 6 to
+// 12 on scores over many magnitudes.  Only rows of one value are slower than a thread
+// per row makes them (50 us for 38), which then never replaces an entry.
 // One CTA per 128-row tile also builds the tile's union list and, for head-packed
 // attention tiles (seg_rows > 0), the lists of its segments of seg_rows tokens.
 constexpr int kRowsMaxC = 1280;   // eight warps' rows fill an SM's shared memory
 constexpr int kRowsTwoC = 704;    // two such CTAs fit
 constexpr int kRowsMinC = 64;
-constexpr int kValueSteps = 14;
+constexpr int kMaxPasses = 128;   // the order holds 2^32 values: at most 3 (32 + 1) + 3 passes
+constexpr float kFar = 60.f;
 
 // order-preserving whole numbers; -0 and +0 share one
 __device__ __forceinline__ uint32_t float_order(float f) {
@@ -577,8 +586,8 @@ __device__ __forceinline__ float row_sum(float v) {   // over a row's eight lane
 struct TailGuess {
     float z, inv_density;
 };
-__device__ __forceinline__ TailGuess tail_guess(int n, int K) {
-    const float f = 1.f / static_cast<float>(n);
+__device__ __forceinline__ TailGuess tail_guess(float n, int K) {
+    const float f = 1.f / n;
     const float z = 1.41421356f * erfinvf(1.f - 2.f * static_cast<float>(K) * f);
     return {z, 2.50662827f * fast_exp2(0.72134752f * z * z) * f};
 }
@@ -620,7 +629,7 @@ __global__ void __launch_bounds__(512, 2) select_rows_kernel(SelParams p, int ve
             for (int m = sub; m < Ci; m += 8) cp_async4(x + m, src + m);
         }
         cp_async_commit();
-        if (Ci != gC && Ci > K) tg = tail_guess(Ci, K);
+        if (Ci != gC && Ci > K) tg = tail_guess(static_cast<float>(Ci), K);
         gC = Ci;
         const int groups = (Ci + 31) >> 5;
         cp_async_wait<0>();
@@ -664,61 +673,105 @@ __global__ void __launch_bounds__(512, 2) select_rows_kernel(SelParams p, int ve
         if (Ci > K) {
             const int ns = min(Ci, 128);
             float sum = 0.f, sq = 0.f;
+            int far = 0;
+            auto sample = [&](float v, bool in) {
+                const float dv = v - mx;
+                const bool near = in && dv > -kFar;   // (NaN: an infinite maximum)
+                far += in && !near ? 1 : 0;
+                const float u = near ? dv : 0.f;
+                sum += u;
+                sq = fmaf(u, u, sq);
+            };
             for (int j = 0; 32 * j < ns; ++j) {
                 const float4 v = xv[8 * j];
                 const int m = 32 * j + 4 * sub;
-                const float d0 = m < ns ? v.x - mx : 0.f, d1 = m + 1 < ns ? v.y - mx : 0.f;
-                const float d2 = m + 2 < ns ? v.z - mx : 0.f, d3 = m + 3 < ns ? v.w - mx : 0.f;
-                sum += (d0 + d1) + (d2 + d3);
-                sq += fmaf(d0, d0, d1 * d1) + fmaf(d2, d2, d3 * d3);
+                sample(v.x, m < ns);
+                sample(v.y, m + 1 < ns);
+                sample(v.z, m + 2 < ns);
+                sample(v.w, m + 3 < ns);
             }
-            const float inv_ns = 1.f / static_cast<float>(ns);
-            const float mean = row_sum(sum) * inv_ns;
-            const float sd = sqrtf(fmaxf(fmaf(-mean, mean, row_sum(sq) * inv_ns), 0.f));
-            uint32_t khi = float_order(mx) + 1u;   // no block there, Ci at lo
-            hi = mx < CUDART_INF_F ? order_float(khi) : mx;
+            float n_near = static_cast<float>(ns);
+            TailGuess g = tg;
+            bool guessed = true;
+            if (__any_sync(0xffffffffu, far > 0)) {
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) far += __shfl_xor_sync(0xffffffffu, far, o);
+                if (far > 0) {
+                    n_near = static_cast<float>(ns - far);
+                    const float n = static_cast<float>(Ci) * n_near / static_cast<float>(ns);
+                    guessed = static_cast<float>(K) < 0.9f * n;
+                    if (guessed) g = tail_guess(n, K);
+                }
+            }
+            const float inv = __fdividef(1.f, n_near);
+            const float mean = row_sum(sum) * inv;
+            const float sd = sqrtf(fmaxf(fmaf(-mean, mean, row_sum(sq) * inv), 0.f));
             above = false;
+            // the K-th largest score lies in [lo, top]: clo scores >= lo, chi > top
+            float top = mx, th = guessed ? mx + mean + sd * g.z : CUDART_NAN_F;
             int clo = Ci, chi = 0;
-            float th = mx + mean + sd * tg.z;
             bool done = false;
 #pragma unroll 1
-            for (int it = 0; it < 64; ++it) {   // at most kValueSteps + 33
-                if (!done && (it >= kValueSteps || !(th > lo && th < hi))) {
-                    const uint32_t klo = float_order(lo);
-                    if (khi - klo <= 1u) {   // only blocks of score lo between the brackets
-                        ties = K - chi;
-                        done = true;
-                    } else {
-                        th = order_float(klo + ((khi - klo) >> 1));
-                    }
+            for (int it = 0; it < kMaxPasses; ++it) {
+                if (!(th > lo && th <= top)) {   // between them
+                    const uint32_t klo = float_order(lo), span = float_order(top) - klo;
+                    th = th > top ? top : order_float(klo + (th <= lo ? 1u : (span >> 1) + (span & 1u)));
                 }
-                if (__all_sync(0xffffffffu, done)) break;
                 int c = 0;
+                float up = CUDART_INF_F, dn = -CUDART_INF_F;
+                auto see = [&](float v) {
+                    if (v >= th) {
+                        ++c;
+                        up = fminf(up, v);
+                    } else {
+                        dn = fmaxf(dn, v);
+                    }
+                };
 #pragma unroll 4
                 for (int j = 0; j < groups; ++j) {
                     const float4 w = xv[8 * j];
-                    c += (w.x >= th ? 1 : 0) + (w.y >= th ? 1 : 0) + (w.z >= th ? 1 : 0) + (w.w >= th ? 1 : 0);
+                    see(w.x);
+                    see(w.y);
+                    see(w.z);
+                    see(w.w);
                 }
 #pragma unroll
                 for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+                float next = c > K ? up : -dn;
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) next = fminf(next, __shfl_xor_sync(0xffffffffu, next, o));
                 if (!done) {
                     if (c > K) {
-                        lo = th;
+                        lo = next;
                         clo = c;
                     } else {
                         hi = th;
-                        khi = float_order(th);
-                        chi = c;
                         above = true;
-                        done = c == K;
+                        top = -next;
+                        chi = c;
+                        if (c == K - 1) lo = top;
                     }
-                    if (it == 0 || clo == Ci)   // Newton on a normal tail count, until something is known below
-                        th += static_cast<float>(c - K - (it > 0 ? 1 : 0)) * sd * tg.inv_density;
-                    else if (it % 3 == 2)
-                        th = 0.5f * (lo + hi);
-                    else
-                        th = lo + (hi - lo) * __fdividef(static_cast<float>(clo - K), static_cast<float>(clo - chi));
+                    if (c == K) {
+                        done = true;
+                    } else if (lo >= top) {   // one value left
+                        ties = K - chi;
+                        done = true;
+                    } else if (clo == K + 1) {   // all but the least
+                        th = order_float(float_order(lo) + 1u);
+                    } else {
+                        const float part = __fdividef(static_cast<float>(clo - K), static_cast<float>(clo - chi));
+                        if (guessed && (it == 0 || (it < 3 && clo == Ci))) {   // Newton on a normal tail count
+                            th += static_cast<float>(c - K - (it > 0 ? 1 : 0)) * sd * g.inv_density;
+                        } else if (guessed && it < 3) {
+                            th = fmaf(top - lo, part, lo);
+                        } else {
+                            const uint32_t klo = float_order(lo), span = float_order(top) - klo;
+                            th = order_float(klo + (it % 3 == 2 ? (span >> 1) + (span & 1u)
+                                                                : max(1u, static_cast<uint32_t>(static_cast<float>(span) * part))));
+                        }
+                    }
                 }
+                if (__all_sync(0xffffffffu, done)) break;
             }
         }
         // kept blocks in order: the masks of eight 32-block groups, one per lane of the
@@ -1603,9 +1656,9 @@ cudaError_t launch_proj(const SelectArgs& a, const SelParams& p, const KernelEnv
 }
 
 // A warp takes its rows one batch of four after another, about 3 us each alone, so
-// sixteen warps where their rows fit several times over (4096 x 8 heads, K = 32: 45.7 us
-// with four warps, 19.9 with sixteen) or where a tile has the SM to itself; else eight
-// (32768 x 8, K = 32: 219 us with four, 207 with eight: 24 warps on an SM for 20).
+// sixteen warps where their rows fit several times over (4096 x 8 heads, K = 32: 41 us
+// with four warps, 21 with sixteen) or where a tile has the SM to itself; else eight
+// (32768 x 8, K = 32: 205 us with four, 196 with eight: 24 warps on an SM for 20).
 int rows_warps(const SelectArgs& a) {
     return a.C <= 128 || (a.C <= 512 && a.BH * a.T <= device_sm_count()) ? 16 : 8;
 }
@@ -1852,15 +1905,15 @@ cudaError_t launch_row_lse(const float* scores, int N, int C, long long rows, fl
     return cudaGetLastError();
 }
 
-// Which kernel selects from given scores (us, thread per row -> eight lanes per row;
-// d = 64, normal scores).  K <= 32: a thread's list is in registers, and up to 2048
-// tokens there is little to replace and its shorter chain wins (2048 x 32 heads, K = 4:
-// 22.9 against 26.7; K = 32: 15.7 / 16.6), from 4096 on the rows kernel (4096 x 8,
-// K = 16: 22.0 / 18.3; 8192 x 2, K = 32: 34.0 / 18.5; 16384 x 4, K = 32: 89.4 / 44.3;
-// 40960 x 2, K = 4: 137 / 97), until its rows leave room for one CTA of eight warps on
-// an SM (81920 x 2, K = 16: 414 / 444).  K > 32: the thread's list is in shared memory
-// and the rows kernel is faster at every length it holds (4096 x 8, K = 64: 23.3 / 15.0;
-// 8192 x 16: 389 / 59; 81920 x 2: 3453 / 475).
+// Which kernel selects from given scores (us by events, thread per row -> eight lanes per
+// row; d = 64, normal scores).  K <= 32: a thread's list is in registers, and up to 2048
+// tokens there is little to replace and its shorter chain holds its own (2048 x 32 heads,
+// K = 4: 27.3 / 24.7; K = 32: 21.4 / 22.5), from 4096 on the rows kernel is faster (4096 x 8,
+// K = 16: 26.9 / 20.5; 8192 x 2, K = 32: 38.8 / 22.8; 16384 x 4, K = 32: 98 / 49;
+// 40960 x 2, K = 4: 144 / 87), until its rows leave room for one CTA of eight warps on
+// an SM (81920 x 2, K = 16: 420 / 409).  K > 32: the thread's list is in shared memory
+// and the rows kernel is faster at every length it holds (4096 x 8, K = 64: 28.6 / 20.9;
+// 8192 x 16: 394 / 62; 81920 x 2: 3456 / 449).
 bool select_builds_segments(const SelectArgs& a) {
     if (a.scores == nullptr || a.score_scale != 1.f || a.full_lse != nullptr) return false;
     return a.topk > 32 ? a.C <= kRowsMaxC : a.C >= kRowsMinC && a.C <= kRowsTwoC;
