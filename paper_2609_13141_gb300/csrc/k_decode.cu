@@ -1013,11 +1013,14 @@ __device__ __forceinline__ uint32_t tc_page_bytes(const int* ent, int e) {
     return ent[2 * e + 1] >= 0 ? 4u * 8192u : 0u;
 }
 
+// Three CTAs an SM at most (shared memory), so 168 registers a thread are there to take:
+// without the second bound the compiler kept to 48, 56 and 64 (G = 1, 2, 4) and spilled
+// (dense lists, 8 sequences of 64K tokens, G = 1, 2, 4: 1235, 640 and 349 us, with it
+// 1194, 625 and 342; a SAS step of one sequence of 8K tokens 19.6 and 19.1).
 template <int G>
-__global__ void __launch_bounds__(kTcThreads) dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK,
-                                                                 const __grid_constant__ CUtensorMap mapV,
-                                                                 DecodeArgs a, int* status, long long limit,
-                                                                 float scale_log2) {
+__global__ void __launch_bounds__(kTcThreads, 3)
+dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV, DecodeArgs a,
+                   int* status, long long limit, float scale_log2) {
     constexpr int D = 128;
     constexpr uint32_t IDESC_S = idesc_bf16(128, 16, 0, 0);
     constexpr uint32_t IDESC_O = idesc_bf16(128, 16, 1, 0);
