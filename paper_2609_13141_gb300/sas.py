@@ -167,11 +167,17 @@ def _ptr(t, dtype, name, required=True):
     return ctypes.c_void_p(t.data_ptr())
 
 
+# The current stream's raw handle without a Stream object; with is_cuda for the device's
+# name in _ptr, the host path of a 256-token layer takes 43 us for 60.  Not a name that
+# torch promises to keep: without it the Stream object is made.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
-    # the raw handle without a Stream object; with is_cuda for the device's name in
-    # _ptr, the host path of a 256-token layer takes 43 us for 60
     if stream is None:
-        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+        if _raw_stream is not None:
+            return ctypes.c_void_p(_raw_stream(torch.cuda.current_device()))
+        stream = torch.cuda.current_stream()
     return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
 
