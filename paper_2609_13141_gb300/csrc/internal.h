@@ -36,21 +36,16 @@ struct KernelEnv {
     long long limit;    // bounded-wait budget in SM cycles
 };
 
-// ---- tcgen05 GEMM:  C[b] = epi(A[b] @ B[b % b_mod]^T (+ bias)), bf16 out (the MLP).
-// A: [batches][M][K], B: [nb][N][K], C: [batches][M][ldc] (row stride ldc).
-// N and K must be multiples of 64.
+// ---- tcgen05 GEMM:  C = epi(A @ B^T (+ bias)), bf16 out (the MLP).
+// A: [M][K], B: [N][K], C: [M][N].  N and K must be multiples of 64.
 struct GemmProblem {
     const void* A;
     const void* B;
     void* C;
     const void* bias;    // bf16 [N] or nullptr
     int M, N, K;
-    int batches, b_mod;
-    long long c_batch_stride;
-    int ldc;
     int gelu;            // 1: exact-erf GELU epilogue
     int after_gemm;      // 1: A is written by the launch_gemm just before on the stream (launched ahead of its end)
-    int max_ctas;        // persistent grid size cap (0: one per SM)
 };
 cudaError_t launch_gemm(const GemmProblem& p, const KernelEnv& env, const char** err);
 

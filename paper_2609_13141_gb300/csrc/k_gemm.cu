@@ -1,10 +1,9 @@
 // Persistent warp-specialised bf16 GEMM on the 5th-generation tensor cores.
 //
-//   C[b] = epi(A[b] @ B[b % b_mod]^T + bias)        (fp32 accumulate, bf16 out)
+//   C = epi(A @ B^T + bias)        (fp32 accumulate, bf16 out)
 //
 // Used for the dense MLP sublayer (up-projection with an exact-GELU epilogue,
-// then the down-projection) and for the selector's batched per-head query
-// projection.  Design:
+// then the down-projection).  Design:
 //   * one CTA per SM, static round-robin over 128 x BN output tiles, grouped
 //     along M so that concurrently running CTAs share operand tiles in L2;
 //   * warp 0 streams 128x64 A and BNx64 B tiles with TMA (128-byte swizzle)
@@ -65,9 +64,6 @@ struct GemmParams {
     bf16* C;
     const bf16* bias;
     int M, N, K;
-    int batches, b_mod;
-    long long c_batch_stride;
-    int ldc;
     int gelu;
     int early_b;             // launched ahead of the kernel that writes A: B may be loaded before it ends
     int* status;
@@ -84,15 +80,12 @@ constexpr int kGroupM = 16;
 // up-projection than polling, which takes issue slots from the epilogue warps).
 constexpr uint32_t kSuspendNs = 1000;
 
-__device__ __forceinline__ void tile_coords(int t, int m_tiles, int n_tiles, int& b, int& m, int& n) {
-    const int per_batch = m_tiles * n_tiles;
-    b = t / per_batch;
-    const int r = t - b * per_batch;
+__device__ __forceinline__ void tile_coords(int t, int m_tiles, int n_tiles, int& m, int& n) {
     const int group_span = kGroupM * n_tiles;
-    const int g = r / group_span;
+    const int g = t / group_span;
     const int first_m = g * kGroupM;
     const int gsize = min(m_tiles - first_m, kGroupM);
-    const int rr = r - g * group_span;
+    const int rr = t - g * group_span;
     m = first_m + rr % gsize;
     n = rr / gsize;
 }
@@ -118,7 +111,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
 
     const int m_tiles = (p.M + kBM - 1) / kBM;
     const int n_tiles = p.N / BN;
-    const int total = p.batches * m_tiles * n_tiles;
+    const int total = m_tiles * n_tiles;
     const int kblocks = p.K / kBK;
 
     if (threadIdx.x == 0) {
@@ -154,14 +147,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
         bool ok = true;
         if (p.early_b) pdl_wait();
         for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-            int b, m, n;
-            tile_coords(t, m_tiles, n_tiles, b, m, n);
+            int m, n;
+            tile_coords(t, m_tiles, n_tiles, m, n);
             for (int kb = 0; kb < kblocks; ++kb) {
                 if (!mbar_wait(&empty_bar[s], ph ^ 1u, wc, kSuspendNs)) { ok = false; break; }
                 uint8_t* sa = smem + s * Cfg::STAGE_BYTES;
                 mbar_arrive_expect_tx(&full_bar[s], Cfg::STAGE_BYTES);
-                tma_load_3d(sa, &mapA, &full_bar[s], kb * kBK, m * kBM, b);
-                tma_load_3d(sa + Cfg::A_BYTES, &mapB, &full_bar[s], kb * kBK, n * BN, b % p.b_mod);
+                tma_load_3d(sa, &mapA, &full_bar[s], kb * kBK, m * kBM, 0);
+                tma_load_3d(sa + Cfg::A_BYTES, &mapB, &full_bar[s], kb * kBK, n * BN, 0);
                 ++issued;
                 if (++s == Cfg::STAGES) { s = 0; ph ^= 1u; }
             }
@@ -219,8 +212,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
             const uint32_t aph = (it >> 1) & 1;
             if (!mbar_wait_warp(&tfull_bar[acc], aph, wc, kSuspendNs)) break;
             tc_fence_after();
-            int b, m, n;
-            tile_coords(t, m_tiles, n_tiles, b, m, n);
+            int m, n;
+            tile_coords(t, m_tiles, n_tiles, m, n);
 #pragma unroll 1
             for (int cg = 0; cg < BN / 64; ++cg, ++nst) {
                 uint8_t* buf = staging + (nst & 1) * 4096;
@@ -262,7 +255,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CU
                 __syncwarp();
                 // rows past M are clipped by the tensor store
                 if (lane == 0) {
-                    tma_store_3d(&mapC, buf, n * BN + cg * 64, m * kBM + q * 32, b);
+                    tma_store_3d(&mapC, buf, n * BN + cg * 64, m * kBM + q * 32, 0);
                     bulk_commit();
                 }
             }
@@ -423,7 +416,7 @@ gemm_split_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constan
             if (p.gelu) {
                 v.x = gelu_erf(v.x); v.y = gelu_erf(v.y); v.z = gelu_erf(v.z); v.w = gelu_erf(v.w);
             }
-            *reinterpret_cast<uint2*>(p.C + static_cast<long long>(m * kBM + r) * p.ldc + n * BN + c) =
+            *reinterpret_cast<uint2*>(p.C + static_cast<long long>(m * kBM + r) * p.N + n * BN + c) =
                 make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
         }
     }
@@ -439,8 +432,7 @@ GemmParams gemm_params(const GemmProblem& p, const KernelEnv& env) {
     gp.C = static_cast<bf16*>(p.C);
     gp.bias = static_cast<const bf16*>(p.bias);
     gp.M = p.M; gp.N = p.N; gp.K = p.K;
-    gp.batches = p.batches; gp.b_mod = p.b_mod;
-    gp.c_batch_stride = p.c_batch_stride; gp.ldc = p.ldc; gp.gelu = p.gelu;
+    gp.gelu = p.gelu;
     gp.early_b = p.after_gemm;
     gp.status = env.status; gp.limit = env.limit;
     return gp;
@@ -540,18 +532,13 @@ cudaError_t launch_bn(const GemmProblem& p, const KernelEnv& env, const char** e
         cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(gemm_kernel<BN>), Cfg::SMEM);
         if (e != cudaSuccess) { *err = "cudaFuncSetAttribute(gemm)"; return e; }
     }
-    if (p.ldc != p.N || (p.batches > 1 && p.c_batch_stride != static_cast<long long>(p.M) * p.N)) {
-        *err = "gemm: C must be a dense [batches][M][N] tensor";
-        return cudaErrorInvalidValue;
-    }
     CUtensorMap ma, mb, mc;
-    const int nb = p.b_mod;
-    if (make_tmap_bf16_3d(&ma, p.A, p.K, p.M, p.batches, kBK, kBM) != 0) { *err = "tensor map A"; return cudaErrorInvalidValue; }
-    if (make_tmap_bf16_3d(&mb, p.B, p.K, p.N, nb, kBK, BN) != 0) { *err = "tensor map B"; return cudaErrorInvalidValue; }
-    if (make_tmap_bf16_3d(&mc, p.C, p.N, p.M, p.batches, 64, 32) != 0) { *err = "tensor map C"; return cudaErrorInvalidValue; }
+    if (make_tmap_bf16_3d(&ma, p.A, p.K, p.M, 1, kBK, kBM) != 0) { *err = "tensor map A"; return cudaErrorInvalidValue; }
+    if (make_tmap_bf16_3d(&mb, p.B, p.K, p.N, 1, kBK, BN) != 0) { *err = "tensor map B"; return cudaErrorInvalidValue; }
+    if (make_tmap_bf16_3d(&mc, p.C, p.N, p.M, 1, 64, 32) != 0) { *err = "tensor map C"; return cudaErrorInvalidValue; }
     const GemmParams gp = gemm_params(p, env);
-    const long long tiles = static_cast<long long>(p.batches) * ((p.M + kBM - 1) / kBM) * (p.N / BN);
-    int grid = p.max_ctas > 0 ? p.max_ctas : device_sm_count();
+    const long long tiles = static_cast<long long>((p.M + kBM - 1) / kBM) * (p.N / BN);
+    int grid = device_room().sms;
     if (tiles < grid) grid = static_cast<int>(tiles);
     cudaError_t e = launch_ex(gemm_kernel<BN>, grid, Cfg::SMEM, 1, p.after_gemm != 0, env.stream, ma, mb, mc, gp);
     if (e != cudaSuccess) *err = "gemm launch";
@@ -606,7 +593,7 @@ GemmShape pick_shape(int M, int N, int K, const Room& room) {
 }  // namespace
 
 cudaError_t launch_gemm(const GemmProblem& p, const KernelEnv& env, const char** err) {
-    const GemmShape g = p.batches == 1 && p.ldc == p.N ? pick_shape(p.M, p.N, p.K, device_room()) : GemmShape{p.N % 256 == 0 ? 256 : (p.N % 128 == 0 ? 128 : 64), 0};
+    const GemmShape g = pick_shape(p.M, p.N, p.K, device_room());
     if (g.split > 0) return g.bn == 128 ? launch_split<128>(p, g.split, env, err) : launch_split<64>(p, g.split, env, err);
     switch (g.bn) {
         case 256: return launch_bn<256>(p, env, err);

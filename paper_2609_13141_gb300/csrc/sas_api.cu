@@ -655,16 +655,14 @@ sas_status sas_mlp_fwd(sas_handle* h, const void* X, const void* W1, const void*
     sas::GemmProblem g1{};
     g1.A = X; g1.B = W1; g1.C = h->hidden; g1.bias = b1;
     g1.M = static_cast<int>(T); g1.N = static_cast<int>(F); g1.K = static_cast<int>(D);
-    g1.batches = 1; g1.b_mod = 1; g1.c_batch_stride = 0; g1.ldc = static_cast<int>(F);
-    g1.gelu = 1; g1.max_ctas = 0;
+    g1.gelu = 1;
     cudaError_t e = timed_launch(h, 4, s, [&] { return sas::launch_gemm(g1, env, &err); });
     if (e != cudaSuccess) return cuda_fail(h, e, err);
 
     sas::GemmProblem g2{};
     g2.A = h->hidden; g2.B = W2; g2.C = Y; g2.bias = b2;
     g2.M = static_cast<int>(T); g2.N = static_cast<int>(D); g2.K = static_cast<int>(F);
-    g2.batches = 1; g2.b_mod = 1; g2.c_batch_stride = 0; g2.ldc = static_cast<int>(D);
-    g2.gelu = 0; g2.after_gemm = 1; g2.max_ctas = 0;
+    g2.gelu = 0; g2.after_gemm = 1;
     e = timed_launch(h, 5, s, [&] { return sas::launch_gemm(g2, env, &err); });
     if (e != cudaSuccess) return cuda_fail(h, e, err);
     return SAS_OK;

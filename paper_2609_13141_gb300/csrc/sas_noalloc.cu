@@ -87,15 +87,13 @@ extern "C" sas_status sas_mlp_fwd_noalloc(const void* X, const void* W1, const v
     sas::GemmProblem g1{};
     g1.A = X; g1.B = W1; g1.C = hidden; g1.bias = b1;
     g1.M = static_cast<int>(T); g1.N = static_cast<int>(F); g1.K = static_cast<int>(D);
-    g1.batches = 1; g1.b_mod = 1; g1.c_batch_stride = 0; g1.ldc = static_cast<int>(F);
-    g1.gelu = 1; g1.max_ctas = 0;
+    g1.gelu = 1;
     if (sas::launch_gemm(g1, env, &err) != cudaSuccess) return SAS_ERR_CUDA;
 
     sas::GemmProblem g2{};
     g2.A = hidden; g2.B = W2; g2.C = Y; g2.bias = b2;
     g2.M = static_cast<int>(T); g2.N = static_cast<int>(D); g2.K = static_cast<int>(F);
-    g2.batches = 1; g2.b_mod = 1; g2.c_batch_stride = 0; g2.ldc = static_cast<int>(D);
-    g2.gelu = 0; g2.after_gemm = 1; g2.max_ctas = 0;
+    g2.gelu = 0; g2.after_gemm = 1;
     if (sas::launch_gemm(g2, env, &err) != cudaSuccess) return SAS_ERR_CUDA;
     return SAS_OK;
 }
