@@ -321,7 +321,12 @@ sas_status sas_fill_varlen_tails(sas_handle* h, const sas_tail* tails, int32_t c
  *   W2 bf16 [D, F]; b2 bf16 [D] or NULL; Y bf16 [T, D].
  * D and F must be multiples of 64; T >= 1.  The hidden activation
  * GELU(X W1^T + b1) is kept as a bf16 [T, F] tensor in handle-owned
- * memory, allocated (synchronously) the first time a call needs more. */
+ * memory, allocated (synchronously) the first time a call needs more.
+ * Results repeat bit for bit, and a row of Y does not depend on the other
+ * rows' values or on where in X it stands.  How the sums over D and F are
+ * split (fp32 partial sums, added in a fixed order) follows from T, D, F and
+ * the device, so the last bits of a row may differ between calls of
+ * different T. */
 sas_status sas_mlp_fwd(sas_handle* h,
                        const void* X, const void* W1, const void* b1,
                        const void* W2, const void* b2, void* Y,
@@ -516,7 +521,12 @@ sas_status sas_decode_summarize(sas_decode_handle* h, const void* K_cache, const
  * In dense mode Wq, Wk and Ksum are not used (may be NULL) and sel_idx must be
  * NULL.  Three kernel launches, one per step above (two in dense mode), each
  * started early by programmatic dependent launch; no allocation, no
- * synchronisation, so the call can be captured in a CUDA graph. */
+ * synchronisation, so the call can be captured in a CUDA graph.
+ * Results repeat bit for bit, and a sequence's do not depend on the other
+ * sequences' tokens or lengths.  How many pages one block of the attention
+ * sums before the partial results are merged follows from the handle's sizes
+ * (with d = 128: B * Hkv groups, topk, the device), so the last bits of O and
+ * LSE may differ between handles of different B; sel_idx does not. */
 sas_status sas_decode_step(sas_decode_handle* h, const void* q, const void* k_new, const void* v_new,
                            void* K_cache, void* V_cache, const int32_t* block_table, const int32_t* seq_lens,
                            const void* Wq, const void* Wk, void* Ksum, void* O, float* LSE, int32_t* sel_idx,
