@@ -8,11 +8,12 @@
 //   dec_score_kernel   s_m = q~ . K~_m / sqrt(d_sel) for the C historical blocks
 //                      (Alg. 2 step 1), CTAs of 256 blocks whose summary rows are
 //                      staged in shared memory by bulk async copies.  Each CTA keeps
-//                      the exact Top-K of its own blocks (rank by counting); the
-//                      last CTA of a group selects the Top-K of those candidates
-//                      (step 2) on the scores' order-preserving bit patterns, by
-//                      counting ranks or, past 512 candidates, a radix select, ties to
-//                      the lower block, and writes the kept list in ascending order.
+//                      the exact Top-K of its own blocks (ranks by counting, past
+//                      kRankRows blocks a sort); the last CTA of a group selects the
+//                      Top-K of those candidates (step 2) on the scores' order-
+//                      preserving bit patterns, by counting ranks or, past kRankMax
+//                      candidates, a radix select, ties to the lower block, and
+//                      writes the kept list in ascending order.
 //   dec_attn_tc_kernel split-KV attention over B_0 and the kept blocks (steps 3-4),
 //                      d = 128: each CTA takes a few pages (K and V slices of 16 KB,
 //                      TMA into a ring), two pages a step on the tensor cores, and
@@ -26,7 +27,7 @@
 // predecessor's results (barrier set-up, reading lengths and queries, the block
 // summaries, the page of the current block) and then waits on the grid dependency.
 // A decode step moves bytes, not flops, and is bound by latencies: at 8 sequences
-// of 64K tokens (8 KV heads, K = 32) 39.8 us a step, against 12.6 us for its bytes.
+// of 64K tokens (8 KV heads, K = 32) 36 us a step, against 12.6 us for its bytes.
 #include <math_constants.h>
 
 #include "internal.h"
@@ -278,7 +279,7 @@ __host__ __device__ inline ScoreSmem score_smem_layout(int nsplit, int topk, int
     L.xchg = L.misc + 64;         // 256 order keys
     L.scan = L.xchg + 256 * 4;    // 16 ints
     L.hist = L.scan + 128;        // 4096 ints of the radix select; kept for every size: two CTAs an
-                                  // SM run a step of 8 x 64K in 39.8 us, three (without them) in 44.3
+                                  // SM ran a step of 8 x 64K (36 us now) in 39.8 us, three (without them) in 44.3
     L.total = L.hist + 4096 * 4;
     return L;
 }
@@ -338,7 +339,8 @@ __device__ __forceinline__ int rank_of(const uint32_t* keys, int M, uint32_t key
 // Exact Top-K of at most kRankMax candidates in ascending block order by counting
 // each one's rank (M^2 comparisons, about 1 us at 160 candidates, against 4 us of the
 // radix select's three histogram passes; two candidates a thread lose: one sequence of
-// 205325 tokens, 416 candidates: 28.2 us against 17.5 for the radix select); same arguments as select_candidates.
+// 205325 tokens, 416 candidates: 28.2 us against 17.5 for the radix select); same
+// arguments as select_candidates.
 __device__ __forceinline__ void select_by_rank(const DecodeArgs& a, int bh, int M, const uint32_t* keys, const int32_t* idx,
                                int* scan) {
     const int K = a.topk, t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -1421,8 +1423,9 @@ cudaError_t launch_attn_tc(const DecodeArgs& a, const KernelEnv& env) {
     if (make_tmap_bf16_3d(&mk, a.K_cache, 128, kBlk, rows, 64, kBlk) != 0) return cudaErrorInvalidValue;
     if (make_tmap_bf16_3d(&mv, a.V_cache, 128, kBlk, rows, 64, kBlk) != 0) return cudaErrorInvalidValue;
     dim3 grid(a.nsplit_a, a.B * a.Hkv);
-    return launch_dependent(a.cluster ? a.nsplit_a : 1, dec_attn_tc_kernel<G>, grid, dim3(kTcThreads), tc_layout(a.nst, a.bpc).total, env.stream,
-                            mk, mv, a, env.status, env.limit, a.sm_scale * kLog2e);
+    return launch_dependent(a.cluster ? a.nsplit_a : 1, dec_attn_tc_kernel<G>, grid, dim3(kTcThreads),
+                            tc_layout(a.nst, a.bpc).total, env.stream, mk, mv, a, env.status, env.limit,
+                            a.sm_scale * kLog2e);
 }
 
 template <int D>
@@ -1517,13 +1520,12 @@ void decode_attn_split(int max_len, int d, bool dense, int groups, int G, int sm
     int per;
     *cluster = 0;
     if (d == 128 && !dense) {
-
         // tensor-core kernel, a SAS list (at most 65 pages): a cluster of S <= 16 CTAs
         // per group, as many as run at once, merging over distributed shared memory.
         // Three CTAs of one 64 KB stage share an SM, but whole clusters have to find
         // room in a GPC, so the grid stays at 8/3 of the SMs (64 groups of 33 pages:
         // 28.8, 25.7, 23.6, 20.8 and 32.0 us with S = 3, 4, 5, 6 and 7; the device's own
-        // count of clusters that fit stops earlier, 45.4 us a step for 39.8).  One
+        // count of clusters that fit stops earlier, 45.4 us a step for 39.8, now 36).  One
         // CTA per SM or fewer: up to three stages, so that a CTA's own loads overlap, and
         // there the device's count decides (8 groups of 49 pages: thirteen CTAs each do
         // not all find room and take 19.5 us, two waves).  (Before: one page pair per CTA

@@ -14,18 +14,19 @@
 // order is the same as on g because log g = s - LSE), so the Top-K decision
 // never depends on how LSE was rounded.
 //
-// One CTA owns one (batch*head, 128-row tile); one thread owns one row and
-// keeps its running max/sum and its Top-K candidates (registers for K <= 32,
-// a shared-memory column otherwise) with replace-the-worst updates.  Under
+// One CTA owns one (batch*head, 128-row tile).  Under
 // GQA the "head" is a KV group: its G query heads share the selection
 // (Sec. 5.3).  Packed sequences: a tile table (varlen_tiles_kernel) gives each
 // CTA its tile's first row, tile index within its sequence and sequence
 // length, so blocks and causality restart at every sequence.
 //
 // Two score sources:
-//   * scores given: eight lanes per row (select_rows_kernel); short and very long
-//     rows one thread each, 32x32 score sub-tiles staged through shared memory
-//     with coalesced 128-byte row loads;
+//   * scores given: eight lanes per row, which bracket the K-th largest score
+//     (select_rows_kernel); short and very long rows (select_builds_segments has
+//     the lines) one thread each, which keeps its running max/sum and its Top-K
+//     candidates (registers for K <= 32, a shared-memory column otherwise) with
+//     replace-the-worst updates, 32x32 score sub-tiles staged through shared
+//     memory with coalesced 128-byte row loads;
 //   * learned selector: on the tensor cores, one thread first projects the
 //     tile's 128 queries (q~ = Q Wq^T into TMEM; under GQA q~ = Wq_g [q_0; ...;
 //     q_{G-1}], accumulated over G rounds of one head each); the row threads round q~
