@@ -184,7 +184,9 @@ sas_status fail(sas_handle* h, sas_status s, const std::string& msg) {
     return s;
 }
 
+// (The error is reported here, once: left in the runtime it would be the next launch's.)
 sas_status cuda_fail(sas_handle* h, cudaError_t e, const char* what) {
+    cudaGetLastError();
     std::string m = std::string(what ? what : "cuda") + ": " + cudaGetErrorString(e);
     return fail(h, e == cudaErrorMemoryAllocation ? SAS_ERR_OOM : SAS_ERR_CUDA, m);
 }

@@ -51,6 +51,7 @@ sas_status dfail(sas_decode_handle* h, sas_status s, const std::string& msg) {
 }
 
 sas_status dcuda_fail(sas_decode_handle* h, cudaError_t e, const char* what) {
+    cudaGetLastError();   // reported here, once
     std::string m = std::string(what) + ": " + cudaGetErrorString(e);
     return dfail(h, e == cudaErrorMemoryAllocation ? SAS_ERR_OOM : SAS_ERR_CUDA, m);
 }

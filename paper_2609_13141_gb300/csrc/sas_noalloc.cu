@@ -88,14 +88,16 @@ extern "C" sas_status sas_mlp_fwd_noalloc(const void* X, const void* W1, const v
     g1.A = X; g1.B = W1; g1.C = hidden; g1.bias = b1;
     g1.M = static_cast<int>(T); g1.N = static_cast<int>(F); g1.K = static_cast<int>(D);
     g1.gelu = 1;
-    if (sas::launch_gemm(g1, env, &err) != cudaSuccess) return SAS_ERR_CUDA;
+    cudaError_t e = sas::launch_gemm(g1, env, &err);
 
     sas::GemmProblem g2{};
     g2.A = hidden; g2.B = W2; g2.C = Y; g2.bias = b2;
     g2.M = static_cast<int>(T); g2.N = static_cast<int>(D); g2.K = static_cast<int>(F);
     g2.gelu = 0; g2.after_gemm = 1;
-    if (sas::launch_gemm(g2, env, &err) != cudaSuccess) return SAS_ERR_CUDA;
-    return SAS_OK;
+    if (e == cudaSuccess) e = sas::launch_gemm(g2, env, &err);
+    if (e == cudaSuccess) return SAS_OK;
+    cudaGetLastError();   // reported here, once: left in the runtime it would be the next launch's
+    return SAS_ERR_CUDA;
 }
 
 extern "C" sas_status sas_mlp_noalloc_get_device_status(int32_t* out_status) {
