@@ -399,7 +399,9 @@ __device__ __forceinline__ int cluster_size() {
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
     return static_cast<int>(r);
 }
+// (.aligned: a warp's lanes have to arrive together, also after loops of unequal length.)
 __device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 __device__ __forceinline__ uint32_t cluster_map(uint32_t saddr, int rank) {
