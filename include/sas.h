@@ -522,11 +522,9 @@ sas_status sas_decode_summarize(sas_decode_handle* h, const void* K_cache, const
  * NULL.  Three kernel launches, one per step above (two in dense mode), each
  * started early by programmatic dependent launch; no allocation, no
  * synchronisation, so the call can be captured in a CUDA graph.
- * Results repeat bit for bit, and a sequence's do not depend on the other
- * sequences' tokens or lengths.  How many pages one block of the attention
- * sums before the partial results are merged follows from the handle's sizes
- * (with d = 128: B * Hkv groups, topk, the device), so the last bits of O and
- * LSE may differ between handles of different B; sel_idx does not. */
+ * Results repeat bit for bit, and a sequence's are the same in any batch:
+ * they depend neither on the other sequences nor on B (in dense mode the sums
+ * are split by max_blocks, so handles of one max_blocks agree). */
 sas_status sas_decode_step(sas_decode_handle* h, const void* q, const void* k_new, const void* v_new,
                            void* K_cache, void* V_cache, const int32_t* block_table, const int32_t* seq_lens,
                            const void* Wq, const void* Wk, void* Ksum, void* O, float* LSE, int32_t* sel_idx,

@@ -184,12 +184,14 @@ struct DecodeArgs {
     int* cnt_attn;              // [B*Hkv]
     int nsplit_s;               // score CTAs per group (kDecScoreChunk blocks each)
     int nsplit_a, bpc, nst;     // attention CTAs per group, list entries per CTA, ring stages
-    int cluster;                // 1: a group's attention CTAs form one cluster and merge among themselves
+    int cluster;                // 1: a group's attention CTAs form one cluster; partials per page pair, merged in order
 };
 constexpr int kDecScoreChunk = 256;
 // Attention split for `groups` lists of at most max_len entries, G query heads each, on sms SMs.
 void decode_attn_split(int max_len, int d, bool dense, int groups, int G, int sms, int* nsplit, int* bpc, int* nst,
                        int* cluster);
+// Floats of `part` a group takes.
+size_t decode_part_floats(const DecodeArgs& a);
 // Dynamic shared memory the score and attention kernels need.
 size_t decode_score_smem(int nsplit, int topk, int d_sel);
 size_t decode_attn_smem(int d, int G, int nst, int bpc);

@@ -16,11 +16,12 @@
 //                      writes the kept list in ascending order.
 //   dec_attn_tc_kernel split-KV attention over B_0 and the kept blocks (steps 3-4),
 //                      d = 128: each CTA takes a few pages (K and V slices of 16 KB,
-//                      TMA into a ring), two pages a step on the tensor cores, and
-//                      keeps an online softmax per head.  A SAS list's CTAs form a
-//                      cluster and merge their partial (max, sum, output) triples
-//                      over distributed shared memory; a dense list's last CTA merges
-//                      them from global memory.
+//                      TMA into a ring), two pages a step on the tensor cores.  A SAS
+//                      list's CTAs form a cluster; every page pair leaves its own
+//                      partial (max, sum, output) and the cluster merges them in list
+//                      order, so that the result does not depend on how many CTAs a
+//                      batch leaves for a list.  A dense list's CTA keeps an online
+//                      softmax over its pages and the last CTA merges.
 //   dec_attn_kernel    the same for d = 64 on the CUDA cores.
 // The three kernels are chained with programmatic dependent launch: each one
 // starts while its predecessor runs, does the work that needs none of the
@@ -970,14 +971,17 @@ __global__ void __launch_bounds__(kAttnThreads) dec_attn_kernel(DecodeArgs a, in
 // written by four 64 x 64 TMA boxes each (page 0 in rows 0-63, page 1 in
 // rows 64-127); Q is [d half][16][128 B], P [key half][16][128 B], both
 // swizzled by the threads that write them.  Every step's O^T is a fresh
-// accumulator that the threads fold into registers (thread t owns row d = t)
-// with the online-softmax rescale.
+// accumulator (thread t owns row d = t): a dense list's threads fold it into
+// registers with the online-softmax rescale, a SAS list's store it as the pair's
+// partial (2.2 KB a step at G = 4, merged from L2; the sums are stored while PV
+// runs, the output behind the next loads).
 
 constexpr int kTcThreads = 128;
 constexpr int kTcTile = 2 * 128 * 128;          // bytes of one K (or V) tile of a step
 constexpr int kTcStage = 2 * kTcTile;           // K and V
 constexpr uint32_t kTcTmemCols = 64;            // S^T in columns 0-15, O^T in 32-47
 constexpr int kMaxDecCluster = 16;              // needs the non-portable cluster size attribute
+constexpr int kPairFloats = 136;                // partial of a page pair and head: max, -, -, -, sum of each warp, output
 
 struct TcLayout {
     size_t q, p, red, alpha, lsum, bars, misc, ent, total;
@@ -1019,7 +1023,7 @@ __device__ __forceinline__ uint32_t tc_page_bytes(const int* ent, int e) {
 // without the second bound the compiler kept to 48, 56 and 64 (G = 1, 2, 4) and spilled
 // (dense lists, 8 sequences of 64K tokens, G = 1, 2, 4: 1235, 640 and 349 us, with it
 // 1194, 625 and 342; a SAS step of one sequence of 8K tokens 19.6 and 19.1).
-template <int G>
+template <int G, bool SAS>
 __global__ void __launch_bounds__(kTcThreads, 3)
 dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_constant__ CUtensorMap mapV, DecodeArgs a,
                    int* status, long long limit, float scale_log2) {
@@ -1063,7 +1067,7 @@ dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         // the current block (entry 0) was appended by the prep kernel, which the
         // score kernel waited for before letting this grid start, so its page can
         // load now (dense mode: the prep kernel precedes this one directly)
-        if (!bad && blockIdx.x == 0 && !a.dense) {
+        if (SAS && !bad && blockIdx.x == 0) {
             int page = __ldg(a.block_table + static_cast<size_t>(b) * a.max_blocks + c);
             if (page < 0 || page >= a.num_pages) page = -1;   // recorded by the prep kernel
             ent[0] = c;
@@ -1086,15 +1090,16 @@ dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         *reinterpret_cast<uint4*>(ps + h * 2048 + row * 128 + (ch << 4)) = make_uint4(0, 0, 0, 0);
     }
     grid_dep_wait();   // the kept list
-    const int L = bad ? 0 : (a.dense ? c : __ldg(a.list_n + bh)) + 1;
-    // a cluster shares its list's pages evenly (a short history has fewer than bpc a CTA)
-    const int per = a.cluster ? (L + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x) : a.bpc;
+    const int L = bad ? 0 : (SAS ? __ldg(a.list_n + bh) : c) + 1;
+    // a cluster shares its list's page pairs evenly (a short history has fewer than bpc / 2 a CTA)
+    const int pairs = (L + 1) >> 1;
+    const int per = SAS ? 2 * ((pairs + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x)) : a.bpc;
     const int j0 = blockIdx.x * per;
     const int cnt = bad ? 0 : max(0, min(j0 + per, L) - j0);
-    const int first = (blockIdx.x == 0 && !a.dense) ? 1 : 0;   // entries set up before the wait
+    const int first = SAS && blockIdx.x == 0 ? 1 : 0;   // entries set up before the wait
     for (int jj = first + t; jj < cnt; jj += kTcThreads) {
         const int j = j0 + jj;
-        const int blk = j == 0 ? c : (a.dense ? j - 1 : __ldg(a.list + static_cast<size_t>(bh) * 64 + j - 1));
+        const int blk = j == 0 ? c : (SAS ? __ldg(a.list + static_cast<size_t>(bh) * 64 + j - 1) : j - 1);
         ent[2 * jj] = blk;
         ent[2 * jj + 1] = block_page(a, b, blk, c, status);
     }
@@ -1117,6 +1122,8 @@ dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         }
     }
 
+    // dense: running maximum, sum and output of this CTA's pages; SAS: of one page pair,
+    // stored before the next
     float m_run[G], l_part[G], o[G];
 #pragma unroll
     for (int h = 0; h < G; ++h) {
@@ -1124,6 +1131,37 @@ dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         l_part[h] = 0.f;
         o[h] = 0.f;
     }
+    float* pair_part = a.part + (static_cast<size_t>(bh) * a.nsplit_a * (a.bpc >> 1) + (j0 >> 1)) * G * kPairFloats;
+    // the CTA's x-th pair: maximum and sum, while the second product runs, then the output
+    auto store_sums = [&](int x) {
+        // warp sums with warp_sum's pairs of lanes, the heads shared out on the way:
+        // a lane ends with head (lane's top log2(G) bits)
+        float v[G];
+#pragma unroll
+        for (int h = 0; h < G; ++h) v[h] = l_part[h];
+        int o = 16;
+#pragma unroll
+        for (int half = G / 2; half > 0; half >>= 1, o >>= 1) {
+            const bool upper = (lane & o) != 0;
+#pragma unroll
+            for (int i = 0; i < half; ++i) {
+                const float send = upper ? v[i] : v[i + half];
+                v[i] = (upper ? v[i + half] : v[i]) + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        }
+#pragma unroll
+        for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+        float* px = pair_part + x * G * kPairFloats;
+        if (lane % (32 / G) == 0) px[lane / (32 / G) * kPairFloats + 4 + warp] = v[0];
+        if (t == 0) {
+#pragma unroll
+            for (int h = 0; h < G; ++h) px[h * kPairFloats] = m_run[h];
+        }
+    };
+    auto store_output = [&](int x) {
+#pragma unroll
+        for (int h = 0; h < G; ++h) pair_part[(x * G + h) * kPairFloats + 8 + t] = o[h];
+    };
     const uint32_t lane_base = tmem + (static_cast<uint32_t>(warp * 32) << 16);
     bool ok = true;
     int j = 0;
@@ -1189,10 +1227,10 @@ dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
 #pragma unroll
         for (int h = 0; h < G; ++h) {
             const float mb = fmaxf(fmaxf(red[h], red[16 + h]), fmaxf(red[32 + h], red[48 + h]));
-            const float m_new = fmaxf(m_run[h], mb);
-            alpha[h] = m_run[h] == -CUDART_INF_F ? 0.f : fast_exp2(m_run[h] - m_new);
+            const float m_new = SAS ? mb : fmaxf(m_run[h], mb);
+            alpha[h] = SAS || m_run[h] == -CUDART_INF_F ? 0.f : fast_exp2(m_run[h] - m_new);
             const float pr = z[h] == -CUDART_INF_F ? 0.f : fast_exp2(z[h] - m_new);
-            l_part[h] = l_part[h] * alpha[h] + pr;
+            l_part[h] = SAS ? pr : l_part[h] * alpha[h] + pr;
             m_run[h] = m_new;
             const int kh = key >> 6, ch = (key & 63) >> 3;
             *reinterpret_cast<bf16*>(ps + kh * 2048 + h * 128 + ((ch ^ (h & 7)) << 4) + ((key & 7) << 1)) =
@@ -1216,6 +1254,7 @@ dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
             __syncwarp();
             pending = 2;
         }
+        if (SAS) store_sums(j);
         if (!mbar_wait_drain(pv_bar, j & 1, limit, status)) ok = false;
         ok = __all_sync(0xffffffffu, ok);
         if (ok) {
@@ -1225,7 +1264,8 @@ dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
             tmem_ld16(lane_base + 32, orr);
             tmem_wait_ld();
 #pragma unroll
-            for (int h = 0; h < G; ++h) o[h] = fmaf(o[h], alpha[h], __uint_as_float(orr[h]));
+            for (int h = 0; h < G; ++h)
+                o[h] = SAS ? __uint_as_float(orr[h]) : fmaf(o[h], alpha[h], __uint_as_float(orr[h]));
             tc_fence_before();
         }
         // (a warp that gave up here says so at the next step's barrier)
@@ -1240,6 +1280,7 @@ dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
             if (e1 < cnt) SAS_TC_LOAD(e1);
             ++issued;
         }
+        if (SAS && ok) store_output(j);
     }
     if (!__syncthreads_and(ok)) {
         // let the tensor cores and the copies in flight finish before leaving
@@ -1254,6 +1295,11 @@ dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
             l_part[h] = 0.f;
             o[h] = 0.f;
         }
+        if (SAS)
+            for (int x = 0; x < steps; ++x) {
+                store_sums(x);
+                store_output(x);
+            }
     }
     tc_fence_before();
     __syncthreads();
@@ -1262,6 +1308,63 @@ dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         tmem_dealloc(tmem, kTcTmemCols);
     }
 
+    if constexpr (SAS) {
+        // the group's CTAs are one cluster: with every pair's partial stored, warp w of
+        // CTA r merges heads r + S w, ... over the list's pairs in order (a lane takes
+        // four of the output's columns).  Short rolled code: it runs once a CTA, so its
+        // instructions come from L2 (unrolled over heads and pairs it took 2 to 7 us)
+        cluster_sync();
+        const int S = cluster_size();
+        constexpr int kBatch = 17;   // pairs of 33 pages
+        const float* base = a.part + static_cast<size_t>(bh) * a.nsplit_a * (a.bpc >> 1) * G * kPairFloats;
+#pragma unroll 1
+        for (int h = cluster_rank() + warp * S; h < G && !bad; h += (kTcThreads / 32) * S) {
+            const float* ph = base + h * kPairFloats;
+            // lane x: maximum and sum of pairs x and 32 + x (a list has at most 33)
+            float w[2] = {-CUDART_INF_F, -CUDART_INF_F}, l[2] = {0.f, 0.f};
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int x = 32 * i + lane;
+                if (x < pairs) {
+                    const float* px = ph + x * G * kPairFloats;
+                    w[i] = __ldcg(px);
+                    const float4 l4 = __ldcg(reinterpret_cast<const float4*>(px + 4));
+                    l[i] = l4.x + l4.y + l4.z + l4.w;
+                }
+            }
+            float M = 0.f, ls = 0.f;
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+            for (int x0 = 0; x0 < pairs; x0 += kBatch) {
+                float4 v[kBatch];
+#pragma unroll
+                for (int x = 0; x < kBatch; ++x)
+                    v[x] = x0 + x < pairs ? __ldcg(reinterpret_cast<const float4*>(ph + (x0 + x) * G * kPairFloats + 8) + lane)
+                                          : make_float4(0.f, 0.f, 0.f, 0.f);
+                if (x0 == 0) {
+                    M = warp_max(fmaxf(w[0], w[1]));
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) w[i] = w[i] == -CUDART_INF_F ? 0.f : fast_exp2(w[i] - M);
+                }
+#pragma unroll
+                for (int x = 0; x < kBatch; ++x) {
+                    const int xx = x0 + x;
+                    if (xx >= pairs) break;
+                    const float wx = __shfl_sync(0xffffffffu, xx < 32 ? w[0] : w[1], xx & 31);
+                    ls = fmaf(wx, __shfl_sync(0xffffffffu, xx < 32 ? l[0] : l[1], xx & 31), ls);
+                    acc.x = fmaf(wx, v[x].x, acc.x);
+                    acc.y = fmaf(wx, v[x].y, acc.y);
+                    acc.z = fmaf(wx, v[x].z, acc.z);
+                    acc.w = fmaf(wx, v[x].w, acc.w);
+                }
+            }
+            const size_t at = static_cast<size_t>(b) * a.Hq + static_cast<size_t>(g) * G + h;
+            reinterpret_cast<uint2*>(static_cast<bf16*>(a.O) + at * D)[lane] =
+                make_uint2(pack_bf16x2(acc.x / ls, acc.y / ls), pack_bf16x2(acc.z / ls, acc.w / ls));
+            if (a.LSE != nullptr && lane == 0) a.LSE[at] = (M + log2f(ls)) / kLog2e;
+        }
+        return;
+    }
     // partial (max, sum, output) of this CTA per head
 #pragma unroll
     for (int h = 0; h < G; ++h) {
@@ -1269,45 +1372,6 @@ dec_attn_tc_kernel(const __grid_constant__ CUtensorMap mapK, const __grid_consta
         if (lane == 0) lsum[warp * 16 + h] = ls;
     }
     __syncthreads();
-    if (a.cluster) {
-        // the group's CTAs are one cluster: each leaves its partials in its shared
-        // memory (the free stage) and merges the heads h = rank, rank + S, ...
-        float* mine = reinterpret_cast<float*>(smem);   // [G][D + 2]
-#pragma unroll
-        for (int h = 0; h < G; ++h) {
-            if (t == 0) {
-                mine[h * (D + 2)] = m_run[h];
-                mine[h * (D + 2) + 1] = lsum[h] + lsum[16 + h] + lsum[32 + h] + lsum[48 + h];
-            }
-            mine[h * (D + 2) + 2 + t] = o[h];
-        }
-        cluster_sync();
-        const int S = cluster_size();
-        const uint32_t own = smem_u32(mine);
-        for (int h = cluster_rank(); h < G && !bad; h += S) {
-            const uint32_t at = own + h * (D + 2) * 4;
-            float mx[kMaxDecCluster], M = -CUDART_INF_F;
-#pragma unroll
-            for (int x = 0; x < kMaxDecCluster; ++x) {
-                mx[x] = x < S ? dsmem_ld_f(cluster_map(at, x)) : -CUDART_INF_F;
-                M = fmaxf(M, mx[x]);
-            }
-            float ls = 0.f, acc = 0.f;
-#pragma unroll
-            for (int x = 0; x < kMaxDecCluster; ++x) {
-                if (x >= S) break;
-                const float w = mx[x] == -CUDART_INF_F ? 0.f : fast_exp2(mx[x] - M);
-                ls = fmaf(w, dsmem_ld_f(cluster_map(at + 4, x)), ls);
-                acc = fmaf(w, dsmem_ld_f(cluster_map(at + 8 + t * 4, x)), acc);
-            }
-            const size_t orow = (static_cast<size_t>(b) * a.Hq + static_cast<size_t>(g) * G + h) * D;
-            static_cast<bf16*>(a.O)[orow + t] = __float2bfloat16_rn(acc / ls);
-            if (a.LSE != nullptr && t == 0)
-                a.LSE[static_cast<size_t>(b) * a.Hq + static_cast<size_t>(g) * G + h] = (M + log2f(ls)) / kLog2e;
-        }
-        cluster_sync();   // the peers have read this CTA's partials
-        return;
-    }
     float* part = a.part + (static_cast<size_t>(bh) * a.nsplit_a + blockIdx.x) * G * (D + 2);
 #pragma unroll
     for (int h = 0; h < G; ++h) {
@@ -1408,22 +1472,22 @@ cudaError_t launch_attn_dg(const DecodeArgs& a, const KernelEnv& env) {
                             env.limit, a.sm_scale * kLog2e);
 }
 
-template <int G>
+template <int G, bool SAS>
 cudaError_t prepare_attn_tc(const DecodeArgs& a) {
     const size_t smem = tc_layout(a.nst, a.bpc).total;
-    return ensure_smem_attr(reinterpret_cast<const void*>(dec_attn_tc_kernel<G>), smem, false, true);
+    return ensure_smem_attr(reinterpret_cast<const void*>(dec_attn_tc_kernel<G, SAS>), smem, false, true);
 }
 
-template <int G>
+template <int G, bool SAS>
 cudaError_t launch_attn_tc(const DecodeArgs& a, const KernelEnv& env) {
-    cudaError_t e = prepare_attn_tc<G>(a);
+    cudaError_t e = prepare_attn_tc<G, SAS>(a);
     if (e != cudaSuccess) return e;
     CUtensorMap mk, mv;
     const uint64_t rows = static_cast<uint64_t>(a.num_pages) * a.Hkv;
     if (make_tmap_bf16_3d(&mk, a.K_cache, 128, kBlk, rows, 64, kBlk) != 0) return cudaErrorInvalidValue;
     if (make_tmap_bf16_3d(&mv, a.V_cache, 128, kBlk, rows, 64, kBlk) != 0) return cudaErrorInvalidValue;
     dim3 grid(a.nsplit_a, a.B * a.Hkv);
-    return launch_dependent(a.cluster ? a.nsplit_a : 1, dec_attn_tc_kernel<G>, grid, dim3(kTcThreads),
+    return launch_dependent(SAS ? a.nsplit_a : 1, dec_attn_tc_kernel<G, SAS>, grid, dim3(kTcThreads),
                             tc_layout(a.nst, a.bpc).total, env.stream, mk, mv, a, env.status, env.limit,
                             a.sm_scale * kLog2e);
 }
@@ -1432,10 +1496,10 @@ template <int D>
 cudaError_t launch_attn_d(const DecodeArgs& a, const KernelEnv& env) {
     if constexpr (D == 128) {
         switch (a.G) {
-            case 1: return launch_attn_tc<1>(a, env);
-            case 2: return launch_attn_tc<2>(a, env);
-            case 4: return launch_attn_tc<4>(a, env);
-            case 8: return launch_attn_tc<8>(a, env);
+            case 1: return a.dense ? launch_attn_tc<1, false>(a, env) : launch_attn_tc<1, true>(a, env);
+            case 2: return a.dense ? launch_attn_tc<2, false>(a, env) : launch_attn_tc<2, true>(a, env);
+            case 4: return a.dense ? launch_attn_tc<4, false>(a, env) : launch_attn_tc<4, true>(a, env);
+            case 8: return a.dense ? launch_attn_tc<8, false>(a, env) : launch_attn_tc<8, true>(a, env);
         }
     } else {
         switch (a.G) {
@@ -1452,10 +1516,10 @@ template <int D>
 cudaError_t prepare_attn_d(const DecodeArgs& a) {
     if constexpr (D == 128) {
         switch (a.G) {
-            case 1: return prepare_attn_tc<1>(a);
-            case 2: return prepare_attn_tc<2>(a);
-            case 4: return prepare_attn_tc<4>(a);
-            case 8: return prepare_attn_tc<8>(a);
+            case 1: return a.dense ? prepare_attn_tc<1, false>(a) : prepare_attn_tc<1, true>(a);
+            case 2: return a.dense ? prepare_attn_tc<2, false>(a) : prepare_attn_tc<2, true>(a);
+            case 4: return a.dense ? prepare_attn_tc<4, false>(a) : prepare_attn_tc<4, true>(a);
+            case 8: return a.dense ? prepare_attn_tc<8, false>(a) : prepare_attn_tc<8, true>(a);
         }
     } else {
         switch (a.G) {
@@ -1491,10 +1555,10 @@ namespace {
 // Clusters of S attention CTAs (a ring of nst stages, bpc pages each) that the device
 // holds at once; 0 if it cannot say.
 int attn_clusters_at_once(int S, int nst, int bpc, int G) {
-    const void* f = G == 1   ? reinterpret_cast<const void*>(dec_attn_tc_kernel<1>)
-                    : G == 2 ? reinterpret_cast<const void*>(dec_attn_tc_kernel<2>)
-                    : G == 4 ? reinterpret_cast<const void*>(dec_attn_tc_kernel<4>)
-                             : reinterpret_cast<const void*>(dec_attn_tc_kernel<8>);
+    const void* f = G == 1   ? reinterpret_cast<const void*>(dec_attn_tc_kernel<1, true>)
+                    : G == 2 ? reinterpret_cast<const void*>(dec_attn_tc_kernel<2, true>)
+                    : G == 4 ? reinterpret_cast<const void*>(dec_attn_tc_kernel<4, true>)
+                             : reinterpret_cast<const void*>(dec_attn_tc_kernel<8, true>);
     const size_t smem = tc_layout(nst, bpc).total;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -1520,23 +1584,27 @@ void decode_attn_split(int max_len, int d, bool dense, int groups, int G, int sm
     int per;
     *cluster = 0;
     if (d == 128 && !dense) {
-        // tensor-core kernel, a SAS list (at most 65 pages): a cluster of S <= 16 CTAs
-        // per group, as many as run at once, merging over distributed shared memory.
+        // tensor-core kernel, a SAS list (at most 65 pages, taken by pairs): a cluster of
+        // S <= 16 CTAs per group, as many as run at once.
         // Three CTAs of one 64 KB stage share an SM, but whole clusters have to find
         // room in a GPC, so the grid stays at 8/3 of the SMs (64 groups of 33 pages:
         // 28.8, 25.7, 23.6, 20.8 and 32.0 us with S = 3, 4, 5, 6 and 7; the device's own
         // count of clusters that fit stops earlier, 45.4 us a step for 39.8, now 36).  One
         // CTA per SM or fewer: up to three stages, so that a CTA's own loads overlap, and
-        // there the device's count decides (8 groups of 49 pages: thirteen CTAs each do
-        // not all find room and take 19.5 us, two waves).  (Before: one page pair per CTA
-        // and a merge through global memory by the last one to arrive; 64 groups took 2.4
-        // waves and 36.5 us.)
+        // there the device's count decides (8 groups of 49 pages: thirteen CTAs each did
+        // not all find room and took 19.5 us, two waves).  (Before clusters: one page pair
+        // per CTA and a merge by the last one to arrive; 64 groups took 2.4 waves and 36.5
+        // us, now 19.0.  A partial per CTA, kept by online softmax and merged over
+        // distributed shared memory, made the result depend on S: a step of 8 sequences
+        // of 64K tokens 29.3 us against 29.7, 32 of 8K 73 against 77, 4 of 32K 32 against
+        // 25, 1 of 8K 18.5 against 16.4.)
         const int fit = 8 * sms / (3 * (groups > 0 ? groups : 1));
         int S = fit < 1 ? 1 : (fit > kMaxDecCluster ? kMaxDecCluster : fit);
+        const int pairs = (max_len + 1) / 2;
         for (;; --S) {
-            per = (max_len + S - 1) / S;
-            S = (max_len + per - 1) / per;
-            const int steps = (per + 1) / 2;
+            const int steps = (pairs + S - 1) / S;
+            S = (pairs + steps - 1) / steps;
+            per = 2 * steps;
             const bool spread = static_cast<long long>(groups) * S <= sms;
             *nst = spread ? (steps < 3 ? steps : 3) : 1;
             if (S == 1 || !spread || attn_clusters_at_once(S, *nst, per, G) >= groups) break;
@@ -1557,6 +1625,11 @@ void decode_attn_split(int max_len, int d, bool dense, int groups, int G, int sm
     }
     *bpc = per;
     *nsplit = (max_len + per - 1) / per;
+}
+
+size_t decode_part_floats(const DecodeArgs& a) {
+    const size_t splits = static_cast<size_t>(a.nsplit_a) * a.G;
+    return a.cluster ? splits * (a.bpc / 2) * kPairFloats : splits * (a.d + 2);
 }
 
 size_t decode_score_smem(int nsplit, int topk, int d_sel) { return score_smem_layout(nsplit, topk, d_sel).total; }

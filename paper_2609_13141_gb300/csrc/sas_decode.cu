@@ -160,9 +160,7 @@ sas_status sas_decode_create(const sas_decode_config* cfg, sas_decode_handle** o
     if (e == cudaSuccess) e = dalloc(&h->cand_idx, ncand * 4);
     if (e == cudaSuccess) e = dalloc(&h->list, static_cast<size_t>(BH) * 64 * 4);
     if (e == cudaSuccess) e = dalloc(&h->list_n, static_cast<size_t>(BH) * 4);
-    // (a cluster merges its partials in shared memory)
-    if (e == cudaSuccess && !h->cluster)
-        e = dalloc(&h->part, static_cast<size_t>(BH) * h->nsplit_a * G * (c.d + 2) * 4);
+    if (e == cudaSuccess) e = dalloc(&h->part, static_cast<size_t>(BH) * sas::decode_part_floats(base_args(h)) * 4);
     if (e == cudaSuccess) e = dalloc(&h->counters, static_cast<size_t>(BH) * 2 * 4);
     if (e == cudaSuccess) e = cudaMemset(h->counters, 0, static_cast<size_t>(BH) * 2 * 4);
     if (e == cudaSuccess) e = dalloc(&h->status, 16);

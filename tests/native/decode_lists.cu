@@ -55,7 +55,7 @@ extern "C" int decode_lists_attend(const void* q, void* K_cache, void* V_cache, 
     a.max_blocks = max_blocks; a.num_pages = pages; a.dense = 0;
     a.sm_scale = 1.f / sqrtf(static_cast<float>(d));
     sas::decode_attn_split(topk + 1, d, false, 1, G, sas::device_sm_count(), &a.nsplit_a, &a.bpc, &a.nst, &a.cluster);
-    if (!a.cluster && a.nsplit_a * G * (d + 2) > part_floats) return -1;
+    if (sas::decode_part_floats(a) > static_cast<size_t>(part_floats)) return -1;
     a.q = q; a.K_cache = K_cache; a.V_cache = V_cache; a.block_table = table; a.seq_lens = n;
     a.list = list; a.list_n = list_n; a.O = O; a.LSE = LSE; a.part = part; a.cnt_sel = counters; a.cnt_attn = counters + 1;
     const sas::KernelEnv env{nullptr, status, 4000000000LL};

@@ -1,6 +1,6 @@
 """What the bits of a result may depend on.  An MLP row: the sizes of the call, not the
-other rows' values or the row's place in its tile.  A decode output: the handle's sizes,
-not the other sequences' tokens or lengths.  Repeated calls give the same bits."""
+other rows' values or the row's place in its tile.  A decode output: neither the other
+sequences' tokens and lengths nor how many there are.  Repeated calls give the same bits."""
 import pytest
 import torch
 
@@ -57,3 +57,39 @@ def test_decode_sequences_do_not_see_each_other(B, Hq, Hkv, topk):
         assert all(torch.equal(x, y) for x, y in zip(step([n] * B, q), a))
     assert sas.sas_decode_get_device_status(dec.h) == 0
     dec.close()
+
+
+@pytest.mark.parametrize("Hq,Hkv,topk,d,dense", [
+    (32, 8, 32, 128, False), (8, 8, 64, 128, False), (64, 8, 48, 128, False), (16, 8, 7, 128, False),
+    (4, 1, 33, 128, False), (32, 8, 32, 64, False), (32, 8, 0, 128, True),
+])
+def test_decode_output_is_the_same_in_any_batch(Hq, Hkv, topk, d, dense):
+    # 1 to 1024 groups: clusters of up to 16 CTAs down to single ones; sequences that fill
+    # their lists and short ones
+    lens = [64 * 70 + 5, 64 * 40 + 64, 64 * 5 + 1, 17]
+    max_blocks, Bmax = 72, 128
+    pages = max_blocks * len(lens)
+    g = torch.Generator(device=DEV).manual_seed(topk)
+    rnd = lambda *s: torch.randn(*s, generator=g, device=DEV).bfloat16()  # noqa: E731
+    K, V, q = rnd(pages, Hkv, 64, d), rnd(pages, Hkv, 64, d), rnd(len(lens), Hq, d)
+    Wq, Wk = (w.to(DEV) for w in synth.decode_selector_weights(Hkv, Hq // Hkv, d, d, seed=3))
+    table = torch.arange(pages, device=DEV, dtype=torch.int32).view(len(lens), max_blocks)
+    first = None
+    for B in (4, 8, 20, 40, Bmax):
+        rep = [t.repeat(B // 4, *([1] * (t.dim() - 1))).contiguous() for t in (q, table)]
+        n = torch.tensor(lens * (B // 4), dtype=torch.int32, device=DEV)
+        dec = sas.SasDecoder(B, Hq, Hkv, d, topk, max_blocks, pages, d_sel=0 if dense else d, dense=dense)
+        if dense:
+            out = dec.step(rep[0], K, V, rep[1], n)
+        else:
+            ks = torch.zeros(B, Hkv, max_blocks, d, device=DEV, dtype=torch.bfloat16)
+            dec.summarize(K, rep[1], n, Wk, ks)
+            out = dec.step(rep[0], K, V, rep[1], n, None, None, Wq, Wk, ks)
+        torch.cuda.synchronize()
+        assert sas.sas_decode_get_device_status(dec.h) == 0
+        dec.close()
+        out = [t for t in out if t is not None]
+        if first is None:
+            first = out
+        for x, y in zip(out, first):
+            assert torch.equal(x[:4], y[:4]) and torch.equal(x[-4:], y[:4])
